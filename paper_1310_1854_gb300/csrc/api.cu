@@ -886,9 +886,11 @@ int ensure_chunks(vgrid_t *g, int64_t N, int64_t chunks, int slot_bytes) {
 }
 
 // persistent grid size for a trace kernel
-int persistent_blocks(const void *fn, const vgrid_launch &l, int sms, int64_t work_items) {
+int persistent_blocks(const vg::TraceFn &fn, const vgrid_launch &l, int sms, int64_t work_items) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, l.block, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn.fn, l.block, fn.smem(l.block)) != cudaSuccess ||
+        per_sm < 1)
+        per_sm = 1;
     if (l.blocks_per_sm > 0 && l.blocks_per_sm < per_sm) per_sm = l.blocks_per_sm;
     int64_t blocks = (int64_t)per_sm * sms;
     const int64_t need = (work_items * l.lanes_per_ray + l.block - 1) / l.block;
@@ -896,24 +898,24 @@ int persistent_blocks(const void *fn, const vgrid_launch &l, int sms, int64_t wo
     return (int)blocks;
 }
 
-int launch_trace(const void *fn, const vgrid_launch &l, int sms, int64_t total, vg::TraceArgs &a, cudaStream_t s) {
-    if (!fn) return fail(VGRID_ERR_ARG, "no kernel for this precision/mode");
+int launch_trace(const vg::TraceFn &fn, const vgrid_launch &l, int sms, int64_t total, vg::TraceArgs &a, cudaStream_t s) {
+    if (!fn.fn) return fail(VGRID_ERR_ARG, "no kernel for this precision/mode");
     const int blocks = persistent_blocks(fn, l, sms, total);
     void *args[] = {&a};
-    VG_CUDA(cudaLaunchKernel(fn, dim3(blocks), dim3(l.block), args, 0, s));
+    VG_CUDA(cudaLaunchKernel(fn.fn, dim3(blocks), dim3(l.block), args, fn.smem(l.block), s));
     vg::count_launches(1);
     return VGRID_OK;
 }
 
 // resident lanes of a persistent float32 launch
-int64_t resident_lanes(vgrid_t *g, const void *fn, const vgrid_launch &l) {
+int64_t resident_lanes(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l) {
     return (int64_t)persistent_blocks(fn, l, g->sms, INT64_MAX / 16) * l.block / l.lanes_per_ray;
 }
 
 // start records (float32 form, or float64 with fp64) for the set in
 // g->d_set; with the ray order (see vgrid_launch.order) also the
 // permutation, which goes to *order
-int locate_start(vgrid_t *g, const void *fn, const vgrid_launch &l, int64_t N, const int32_t **order, cudaStream_t s,
+int locate_start(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l, int64_t N, const int32_t **order, cudaStream_t s,
                 bool fp64 = false) {
     *order = nullptr;
     const int prep = fp64 ? vg::PREP_FP64 : vg::PREP_FP32;
@@ -960,7 +962,7 @@ int trace_tau_chunk(vgrid_t *g, const double *origin, const double *dir, int64_t
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, reset_stats ? g->d_stats : nullptr, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, ks.fn[row][vg::MODE_TAU], L, n, &order, s, fp64 != 0))) return rc;
+    if ((rc = locate_start(g, ks.get(row, vg::MODE_TAU), L, n, &order, s, fp64 != 0))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.grids = g->d_desc;
@@ -973,7 +975,7 @@ int trace_tau_chunk(vgrid_t *g, const double *origin, const double *dir, int64_t
     a.s1 = set;
     a.order = order;
     mark(g, 1, 0, s);
-    if ((rc = launch_trace(ks.fn[row][vg::MODE_TAU], L, g->sms, n, a, s))) return rc;
+    if ((rc = launch_trace(ks.get(row, vg::MODE_TAU), L, g->sms, n, a, s))) return rc;
     mark(g, 1, 1, s);
     return VGRID_OK;
 }
@@ -989,7 +991,7 @@ int trace_chunk_slot(vgrid_t *g, int k, const double *origin, const double *dir,
     vgrid_launch L = g->launch;
     const int fp64 = precision == VGRID_FP64;
     const int row = precision_row(precision, L);
-    const void *fn = kernels(L.lanes_per_ray).fn[row][vg::MODE_TAU];
+    const vg::TraceFn fn = kernels(L.lanes_per_ray).get(row, vg::MODE_TAU);
     cudaStream_t t = g->s_loc;
     VG_CUDA(cudaStreamWaitEvent(t, g->ev_in[k], 0));
     VG_CUDA(cudaStreamWaitEvent(t, g->ev_k[k], 0));
@@ -1100,7 +1102,7 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
     {
-        const void *fn = ks.fn[row][output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS];
+        const vg::TraceFn fn = ks.get(row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS);
         if ((rc = locate_start(g, fn, L, N, &order, s, fp64 != 0))) return rc;
     }
     mark(g, 0, 1, s);
@@ -1116,7 +1118,7 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     a.s1 = set;
     if (output == VGRID_TAU) {
         mark(g, 1, 0, s);
-        if ((rc = launch_trace(ks.fn[row][vg::MODE_TAU], L, g->sms, N, a, s))) return rc;
+        if ((rc = launch_trace(ks.get(row, vg::MODE_TAU), L, g->sms, N, a, s))) return rc;
         mark(g, 1, 1, s);
         if (stats) return read_stats(g->d_stats, stats, s);
         return VGRID_OK;
@@ -1127,7 +1129,7 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     // fills or starts (at most cap / kSegChunk + min(N, cap) when the total
     // fits the capacity) plus the page each warp may leave unused, so it
     // never runs out when the segments fit the caller's buffers.
-    const void *fn = ks.fn[row][vg::MODE_SEGS];
+    const vg::TraceFn fn = ks.get(row, vg::MODE_SEGS);
     int64_t chunks = 0;
     if (seg_capacity > 0) {
         const int64_t warps = (int64_t)persistent_blocks(fn, L, g->sms, N) * L.block / 32;
@@ -1310,7 +1312,7 @@ int vgrid_trace_grad(vgrid_t *g, const double *origin, const double *dir, int64_
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).fn[0][vg::MODE_GRAD], g->launch, N, &order, s))) return rc;
+    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).get(0, vg::MODE_GRAD), g->launch, N, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
@@ -1325,7 +1327,7 @@ int vgrid_trace_grad(vgrid_t *g, const double *origin, const double *dir, int64_
     a.g1 = g->hd;
     a.s1 = set;
     mark(g, 1, 0, s);
-    rc = launch_trace(kernels(g->launch.lanes_per_ray).fn[0][vg::MODE_GRAD], g->launch, g->sms, N, a, s);
+    rc = launch_trace(kernels(g->launch.lanes_per_ray).get(0, vg::MODE_GRAD), g->launch, g->sms, N, a, s);
     mark(g, 1, 1, s);
     return rc;
 }
@@ -1377,7 +1379,7 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).fn[0][vg::MODE_INTERACT], g->launch, N, &order, s))) return rc;
+    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).get(0, vg::MODE_INTERACT), g->launch, N, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
@@ -1395,7 +1397,7 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
     a.g1 = g->hd;
     a.s1 = set;
     mark(g, 1, 0, s);
-    rc = launch_trace(kernels(g->launch.lanes_per_ray).fn[0][vg::MODE_INTERACT], g->launch, g->sms, N, a, s);
+    rc = launch_trace(kernels(g->launch.lanes_per_ray).get(0, vg::MODE_INTERACT), g->launch, g->sms, N, a, s);
     mark(g, 1, 1, s);
     return rc;
 }
@@ -1506,7 +1508,7 @@ static int batch_issue(vgrid_batch_t *b, cudaStream_t s) {
     a.total = b->total;
     a.queue = b->d_queue;
     a.stats = b->d_stats;
-    return launch_trace(kernels(b->launch.lanes_per_ray).batch, b->launch, b->sms, b->total, a, s);
+    return launch_trace(kernels(b->launch.lanes_per_ray).get_batch(), b->launch, b->sms, b->total, a, s);
 }
 
 int vgrid_batch_run(vgrid_batch_t *b, int use_graph, vgrid_stats *stats, vgrid_stream_t stream) {

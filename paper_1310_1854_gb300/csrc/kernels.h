@@ -49,6 +49,27 @@ struct TraceArgs {
 };
 
 
+// Shared memory of a traversal block, per warp: the queue of rays to start
+// (records, ray indices, head and count, per-ray scalars: the adjoint's
+// dL/dtau, interaction's tau_int and weight, a batch's ray set) and the float32
+// form's per-ray values.
+constexpr int kFetch = 32;    // rays a warp's queue holds
+constexpr int kRayVals = 11;  // per-ray floats of the float32 form
+constexpr int trace_queue_bytes(int mode, bool batch) {
+    return kFetch * ((int)sizeof(RayPrep) + 8 + 4 * (mode == MODE_GRAD ? 1 : mode == MODE_INTERACT ? 2 : 0) +
+                     (batch ? 4 : 0)) + 16;
+}
+constexpr int trace_warp_bytes(bool fp64, int mode, bool batch) {
+    return trace_queue_bytes(mode, batch) + (fp64 ? 0 : 32 * 4 * kRayVals);
+}
+
+// a traversal kernel and the shared memory that a block of it takes per warp
+struct TraceFn {
+    const void *fn;
+    int warp_bytes;
+    size_t smem(int block) const { return (size_t)(block / 32) * warp_bytes; }
+};
+
 // fn[fp64][mode]: single-grid trace kernels of one lanes-per-ray value
 // (nullptr if absent); batch: the float32 tau kernel over many grids
 struct KernelSet {
@@ -56,6 +77,8 @@ struct KernelSet {
     // exact lengths (one lane per ray only)
     const void *fn[3][NUM_MODES];
     const void *batch;
+    TraceFn get(int row, int mode) const { return {fn[row][mode], trace_warp_bytes(row == 1, mode, false)}; }
+    TraceFn get_batch() const { return {batch, trace_warp_bytes(false, MODE_TAU, true)}; }
 };
 
 void kernel_table_lpr1(KernelSet &k);

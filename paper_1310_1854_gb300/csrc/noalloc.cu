@@ -102,9 +102,10 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
             case 8: vg::kernel_table_lpr8(ks); break;
             default: vg::kernel_table_lpr4(ks); break;
         }
-        const void *fn = ks.fn[precision == VGRID_FP32_EXACT ? 2 : fp64][vg::MODE_TAU];
+        const vg::TraceFn fn = ks.get(precision == VGRID_FP32_EXACT ? 2 : fp64, vg::MODE_TAU);
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, v.block, 0) != cudaSuccess || per_sm < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn.fn, v.block, fn.smem(v.block)) != cudaSuccess ||
+            per_sm < 1)
             per_sm = 1;
         if (v.blocks_per_sm > 0 && v.blocks_per_sm < per_sm) per_sm = v.blocks_per_sm;
         int64_t blocks = (int64_t)per_sm * v.sms;
@@ -120,7 +121,7 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
         a.g1 = v.hd;
         a.s1 = set;
         void *args[] = {&a};
-        e = cudaLaunchKernel(fn, dim3((unsigned)blocks), dim3(v.block), args, 0, s);
+        e = cudaLaunchKernel(fn.fn, dim3((unsigned)blocks), dim3(v.block), args, fn.smem(v.block), s);
         if (e != cudaSuccess) rc = fail(VGRID_ERR_CUDA, std::string("cudaLaunchKernel: ") + cudaGetErrorString(e));
     } while (0);
     if (prev != v.device) cudaSetDevice(prev);
