@@ -396,6 +396,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     const float fnan = std::numeric_limits<float>::quiet_NaN();
     // every cell writes only its own blocks and site entry
     vg::parallel_for(M, o.threads, 1 << 12, [&](int64_t i0, int64_t i1) {
+    std::vector<std::pair<double, int32_t>> near;  // cell neighbours by |p_j - p_i|^2
     for (int64_t i = i0; i < i1; i++) {
         const int64_t b = g->cells.off[i], e = g->cells.off[i + 1];
         const float pi[3] = {(float)Si[3 * i + 0], (float)Si[3 * i + 1], (float)Si[3 * i + 2]};
@@ -414,7 +415,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         f[5] = 1.0f;
         put_int(f + 7, (int32_t)boffs[i]);
         double n1max = 0.0;
-        int64_t k = 0;
+        near.clear();
         for (int64_t q = b; q < e; q++) {
             float *r = &blocks[4 * (boffs[i] + 1 + (q - b))];
             const int32_t j = g->cells.idx[q];
@@ -425,19 +426,32 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
                 r[1] = pj[1];
                 r[2] = pj[2];
                 put_int(r + 3, (int32_t)boffs[j]);
-                float *rr = &f[4 * (2 + k++)];
-                double n1 = 0.0;
+                double d2 = 0.0;
                 for (int c = 0; c < 3; c++) {
                     volatile float d = pj[c] - pi[c];  // one float32 rounding, as on the device
-                    rr[c] = d;
-                    n1 += std::fabs((double)rr[c]);
+                    d2 += (double)d * (double)d;
                 }
-                put_int(rr + 3, (int32_t)foffs[j]);
-                n1max = std::max(n1max, n1);
+                near.emplace_back(d2, j);
             } else {
                 r[0] = r[1] = r[2] = 0.0f;
                 put_int(r + 3, j);
             }
+        }
+        // the relative records nearest neighbour first: the exit search stops
+        // once the rest lies too far from the site to be reached
+        std::sort(near.begin(), near.end());
+        int64_t k = 0;
+        for (; k < (int64_t)near.size(); k++) {
+            const int32_t j = near[(size_t)k].second;
+            float *rr = &f[4 * (2 + k)];
+            double n1 = 0.0;
+            for (int c = 0; c < 3; c++) {
+                volatile float d = (float)Si[3 * (int64_t)j + c] - pi[c];
+                rr[c] = d;
+                n1 += std::fabs((double)rr[c]);
+            }
+            put_int(rr + 3, (int32_t)foffs[j]);
+            n1max = std::max(n1max, n1);
         }
         for (; k < c4; k++) {
             float *rr = &f[4 * (2 + k)];

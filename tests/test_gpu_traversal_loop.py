@@ -1,7 +1,8 @@
-"""The traversal loop's ray queue (GPU).
+"""The traversal loop's ray queue and early stop of the exit search (GPU).
 
-The queue hands a warp up to 32 rays at a time: that may not change a result,
-so every comparison is exact (bit for bit).
+The queue hands a warp up to 32 rays at a time and the search leaves out the
+records that lie too far from the site: neither may change a result, so every
+comparison is exact (bit for bit).
 """
 import numpy as np
 import pytest
@@ -45,3 +46,45 @@ def test_queue_hands_out_every_ray_once(lanes, block, per_sm, order):
             assert st["decisions"] == st["crossings"] + st["zero_steps"]  # no step without an exit here
         c, d, _ = vg.interact(O[:n], D[:n], tint[:n], w[:n])
         assert torch.equal(c, cell[:n]) and torch.equal(d, s[:n]), n
+
+
+def _shell(n):
+    k = np.arange(n) + 0.5
+    th, ph = np.arccos(1.0 - 2.0 * k / n), np.pi * (1.0 + 5.0 ** 0.5) * k
+    return np.stack([np.sin(th) * np.cos(ph), np.sin(th) * np.sin(ph), np.cos(th)], axis=1)
+
+
+def _sites(kind, rng):
+    if kind == "few":            # one to three records, all padding behind them
+        return rng.uniform(-1.0, 1.0, (3, 3))
+    if kind == "equidistant":    # a cell whose 80 neighbours are equally far
+        far = rng.uniform(-1.0, 1.0, (1500, 3))
+        return np.concatenate([[[0.0, 0.0, 0.0]], 0.5 * _shell(80), far[np.linalg.norm(far, axis=1) > 0.75][:200]])
+    if kind == "near and far":   # neighbours at distances over eight decades
+        return _shell(120) * (10.0 ** rng.uniform(-8.0, 0.0, 120))[:, None] * 0.99
+    return np.stack(np.meshgrid(*[np.linspace(-0.75, 0.75, 7)] * 3, indexing="ij"), -1).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("kind", ["few", "equidistant", "near and far", "lattice"])
+def test_early_stop_takes_the_same_paths(kind):
+    """One lane per ray stops early, four lanes read every record, the float64
+    form tests every plane in float64."""
+    from paper_1310_1854_gb300 import VoronoiGrid
+    rng = gen.rng_for(43)
+    S = np.unique(np.float32(_sites(kind, rng)).astype(np.float64), axis=0)
+    vg = VoronoiGrid(S, gen.CUBE_BOX)
+    vg.set_density(dev(rng.uniform(0.5, 2.0, len(S)).astype(np.float32)))
+    rays = gen.uniform_rays(4_000, 44)
+    k = rng.integers(0, len(S), 1_000)
+    rays.origin[:1_000] = np.clip(S[k] + 1e-7 * rng.standard_normal((1_000, 3)), -1.0, 1.0)
+    O, D = dev(rays.origin), dev(rays.dir)
+    a = vg.trace(O, D, segments=True, stats=True)
+    vg.set_launch(lanes_per_ray=4)
+    b = vg.trace(O, D, segments=True, stats=True)
+    assert a.stats == b.stats
+    for x in ("tau", "seg_off", "seg_cell", "seg_len"):
+        assert torch.equal(getattr(a, x), getattr(b, x)), x
+    vg.set_launch()
+    c = vg.trace(O, D, precision="fp64", segments=True)
+    if kind != "lattice":        # rays through edges may order ties otherwise
+        assert torch.equal(a.seg_off, c.seg_off) and torch.equal(a.seg_cell, c.seg_cell)
