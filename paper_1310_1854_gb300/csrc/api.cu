@@ -87,7 +87,6 @@ struct vgrid {
     GridDev *d_desc = nullptr;
     float4 *d_site = nullptr;
     float4 *d_cells = nullptr;
-    float4 *d_rec64 = nullptr;       // float64 form: exact differences per entry of d_cells
     float4 *d_rel = nullptr;
     int32_t *d_perm = nullptr;
     int32_t *d_blk_off = nullptr;
@@ -237,7 +236,7 @@ static void free_grid(vgrid_t *g) {
     if (g->d_hhist) cudaFree(g->d_hhist);
     if (g->d_hqueue) cudaFree(g->d_hqueue);
     if (g->d_hset) cudaFree(g->d_hset);
-    void *ptrs[] = {g->d_desc,  g->d_site,  g->d_cells, g->d_rec64, g->d_rel,   g->d_dens,  g->d_bin,   g->d_hist,
+    void *ptrs[] = {g->d_desc,  g->d_site,  g->d_cells, g->d_rel,   g->d_dens,  g->d_bin,   g->d_hist,
                     g->d_order, g->d_perm,  g->d_blk_off, g->d_blk_rec, g->d_queue, g->d_stats, g->d_set,
                     g->d_start, g->d_scan,  g->d_entry, g->d_slots, g->d_chunk_meta, g->d_chunk_inv, g->d_coff, g->d_cursor};
     for (void *p : ptrs)
@@ -537,7 +536,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     }
     VG_ALLOC(g->d_site, M);
     VG_ALLOC(g->d_cells, nrec);
-    VG_ALLOC(g->d_rec64, 2 * (size_t)nrec);
     VG_ALLOC(g->d_rel, nrel);
     VG_ALLOC(g->d_perm, M);
     VG_ALLOC(g->d_blk_off, boff.size());
@@ -614,15 +612,9 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         e = cudaMemcpy(g->d_blk_rec, brec.get(), sizeof(float) * 4 * nbrec, cudaMemcpyHostToDevice);
     }
 
-    if (e == cudaSuccess) {
-        e = vg::launch_build_rec64(g->d_site, g->d_rel, g->d_cells, M, nrec, g->d_rec64, g->sms, 0);
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    }
-
     GridDev &hd = g->hd;
     hd.site = g->d_site;
     hd.cells = g->d_cells;
-    hd.rec64 = g->d_rec64;
     hd.rel = g->d_rel;
     hd.perm = g->d_perm;
     hd.blk_off = g->d_blk_off;

@@ -43,13 +43,16 @@ cudaError_t launch_prepare(RaySetDev *d_set, const RaySetDev &set, unsigned long
 // only, written as the caller's id to out_caller (no start record), with
 // float32 (rechecked) or float64 distances;
 // PREP_FP32: float32 form (cell, direction check, wall exit of Eq. 5 and the
-// float pairs of origin and direction); PREP_FP64: float64 form (cell and
-// direction check). The caller's id of the cell goes to out_caller if given.
+// float pairs of origin and direction); PREP_FP64: float64 form (cell,
+// direction check, bounds on the wall exit, origin and direction). The caller's id of the cell goes to out_caller if given.
+// One instance per kind of record, with the search inlined: the cells alone
+// then fit without spills.
 // Held to five blocks of 256 threads per SM (48 registers, a few spilled):
 // the kernel waits on its loads, and the extra warps hide more of that wait
 // than the spilled bytes cost.
+template <int PREP>
 __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets,
-                                                     int64_t total, int prep, int32_t *out_caller, uint8_t *bin,
+                                                     int64_t total, int32_t *out_caller, uint8_t *bin,
                                                      uint32_t *hist) {
     __shared__ uint32_t s_hist[kOrderBins];
     if (bin) {
@@ -66,9 +69,9 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
         // float32 distances with the proven float64 fallback give exactly the
         // float64 argmin, so both traversal forms start that way; only
         // vgrid_locate's float64 mode (PREP_CELL64) scans in float64
-        int m = locate_point<true>(gp, P, prep != PREP_CELL64, nullptr);
+        int m = locate_point<true>(gp, P, PREP != PREP_CELL64, nullptr);
         if (out_caller) out_caller[w] = m >= 0 ? __ldg(&gp->perm[m]) : -1;
-        if (prep == PREP_CELL32 || prep == PREP_CELL64) continue;
+        if (PREP == PREP_CELL32 || PREP == PREP_CELL64) continue;
         RayPrep *out = rs.start + li;
         const double *d = rs.dir + 3 * li;
         const double k[3] = {__ldg(d), __ldg(d + 1), __ldg(d + 2)};
@@ -94,13 +97,9 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
             unit = fabs(kk - 1.0) <= 2.000001e-6;
         }
         if (!unit) m = -2;
-        const bool fp64 = prep == PREP_FP64;  // the float64 form needs the cell only
-        if (fp64 && !bin) {
-            out->cell = m;
-            continue;
-        }
-        // the float32 traversal starts from the cell's relative block
-        p.cell = m >= 0 && !fp64 ? __float_as_int(__ldg(&gp->site[m]).w) : m;
+        constexpr bool fp64 = PREP == PREP_FP64;
+        // the traversal starts from the cell's relative block
+        p.cell = m >= 0 ? __float_as_int(__ldg(&gp->site[m]).w) : m;
         // distance to the wall ahead (Eq. 5 for the walls the ray faces), as
         // a float pair: q1 = n/k rounded, the exact remainder n - q1 k by
         // fma, then q2 = remainder / k (relative error a few 2^-48); in a
@@ -108,9 +107,18 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
         // split into a float pair
         float th = 3.0e38f, tl = 0.0f;
         int wid = -1;
+        // float64 form: bounds on the exit distance that also hold for what it
+        // evaluates later from its moved point, which is off the line by up to
+        // steps 2^-53 |coordinates| (it trusts them up to 2^15 steps): a wall's
+        // distance then moves by that over |k_c|, the sphere's root, whose
+        // square root may have a small argument, by up to 2^-18 of the scale
+        const float scale = (float)gp->scale;
+        float w_lo = 3.0e38f, w_hi = 3.0e38f, w_lo2 = 3.0e38f;
         if (gp->domain == VGRID_DOMAIN_SPHERE) {
             split_pair(sphere_exit64(gp, P.x, k), th, tl);
             wid = kSphereWall;
+            w_lo = __fsub_rd(th, 0x1p-18f * scale);
+            w_hi = __fadd_ru(th, 0x1p-18f * scale);
         }
         for (int c = 0; c < 3 && gp->domain != VGRID_DOMAIN_SPHERE; c++) {
             const uint64_t kb = dbits(k[c]);
@@ -125,6 +133,17 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
             const float q2 = __fdiv_rn(rem, kh);
             float h, l;
             two_sum(q1, q2, h, l);
+            if (fp64) {
+                const float off = __fmaf_ru(kU, fabsf(h), __fmul_ru(0x1p-36f * scale, __fdiv_ru(1.0f, fabsf(kh))));
+                const float lo = __fsub_rd(h, off), hi = __fadd_ru(h, off);
+                if (lo < w_lo) {
+                    w_lo2 = w_lo;
+                    w_lo = lo;
+                    w_hi = hi;
+                } else {
+                    w_lo2 = fminf(w_lo2, lo);
+                }
+            }
             if (h < th || (h == th && l < tl)) {
                 th = h;
                 tl = l;
@@ -140,11 +159,17 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
         p.wall = wid;
         p.tmax_hi = th;
         p.tmax_lo = tl;
+        float4 *dst = reinterpret_cast<float4 *>(out);
         if (fp64) {
-            out->cell = m;
+            // a NaN bound (from an infinite one) names no wall either
+            const bool one = w_hi < w_lo2 && wid < 0;
+            dst[0] = make_float4(__int_as_float(p.cell), __int_as_float(wid), w_lo,
+                                 one ? w_hi : __int_as_float(0x7f800000));
+            reinterpret_cast<double2 *>(dst)[1] = make_double2(P.x[0], P.x[1]);
+            reinterpret_cast<double2 *>(dst)[2] = make_double2(P.x[2], k[0]);
+            reinterpret_cast<double2 *>(dst)[3] = make_double2(k[1], k[2]);
         } else {
             const float4 *src = reinterpret_cast<const float4 *>(&p);
-            float4 *dst = reinterpret_cast<float4 *>(out);
             for (int q = 0; q < 4; q++) dst[q] = src[q];
         }
         if (bin) {
@@ -182,14 +207,24 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
     }
 }
 
-cudaError_t launch_locate_ordered(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total,
-                                  const RayOrder &ord, int prep, int sms, cudaStream_t s) {
+static cudaError_t launch_locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
+                                        int32_t *out_caller, uint8_t *bin, uint32_t *hist, int sms, cudaStream_t s) {
     if (total <= 0) return cudaSuccess;
-    int64_t blocks = (total + 255) / 256;
-    blocks = blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16;
-    locate_kernel<<<(unsigned)blocks, 256, 0, s>>>(grids, sets, nsets, total, prep, nullptr, ord.bin, ord.hist);
+    const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)sms * 16);
+    const dim3 g((unsigned)blocks);
+    switch (prep) {
+        case PREP_CELL32: locate_kernel<PREP_CELL32><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
+        case PREP_CELL64: locate_kernel<PREP_CELL64><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
+        case PREP_FP64: locate_kernel<PREP_FP64><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
+        default: locate_kernel<PREP_FP32><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
+    }
     count_launches(1);
     return cudaGetLastError();
+}
+
+cudaError_t launch_locate_ordered(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total,
+                                  const RayOrder &ord, int prep, int sms, cudaStream_t s) {
+    return launch_locate_kernel(grids, sets, nsets, total, prep, nullptr, ord.bin, ord.hist, sms, s);
 }
 
 // cursor[b] = number of rays in longer bins (the longest bin goes first)
@@ -251,12 +286,7 @@ cudaError_t launch_order(const RayOrder &ord, int64_t total, int sms, cudaStream
 
 cudaError_t launch_locate(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
                           int32_t *out_caller, int sms, cudaStream_t s) {
-    if (total <= 0) return cudaSuccess;
-    int64_t blocks = (total + 255) / 256;
-    blocks = blocks < (int64_t)sms * 16 ? blocks : (int64_t)sms * 16;
-    locate_kernel<<<(unsigned)blocks, 256, 0, s>>>(grids, sets, nsets, total, prep, out_caller, nullptr, nullptr);
-    count_launches(1);
-    return cudaGetLastError();
+    return launch_locate_kernel(grids, sets, nsets, total, prep, out_caller, nullptr, nullptr, sms, s);
 }
 
 // rho (caller order) into the headers of both forms of the cell blocks
@@ -494,56 +524,6 @@ cudaError_t launch_compact_segments(const int64_t *off, int64_t N, int64_t chunk
     else
         compact_segments_kernel<false><<<grid_for(chunk_cap * kSegChunk, sms), 256, 0, s>>>(off, coff, N, cap, inv,
                                                                                             meta, slots, cell, len);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-// exact float64 sum of two floats? (the TwoSum error term is zero)
-__device__ __forceinline__ bool exact_sum(double a, double b) {
-    const double s = __dadd_rn(a, b), bb = __dsub_rn(s, a);
-    return __dadd_rn(__dsub_rn(a, __dsub_rn(s, bb)), __dsub_rn(b, bb)) == 0.0;
-}
-
-// One thread per cell: the records of its absolute block get n = p_j - p_m
-// in float64 (site coordinates are floats, so n is exact unless their
-// exponents lie far apart; then the flag sends the kernel back to the float
-// coordinates, as it does for p_j + p_m).
-__global__ void build_rec64_kernel(const float4 *site, const float4 *rel, const float4 *cells, int64_t M,
-                                   float4 *rec64) {
-    for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < M; m += (int64_t)gridDim.x * blockDim.x) {
-        const float4 sm = site[m];
-        const int A = __float_as_int(rel[__float_as_int(sm.w) + 1].w);
-        const int cnt = __float_as_int(cells[A].y);
-        rec64[2 * (int64_t)A] = make_float4(0.f, 0.f, 0.f, 0.f);
-        rec64[2 * (int64_t)A + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const double pm[3] = {(double)sm.x, (double)sm.y, (double)sm.z};
-        for (int p = 1; p <= cnt; p++) {
-            const float4 q = cells[A + p];
-            const int w = __float_as_int(q.w);
-            double n[3] = {0.0, 0.0, 0.0};
-            int flag = 0;
-            if (w >= 0) {
-                const double pj[3] = {(double)q.x, (double)q.y, (double)q.z};
-                for (int c = 0; c < 3; c++) {
-                    n[c] = __dsub_rn(pj[c], pm[c]);
-                    if (!exact_sum(pj[c], -pm[c]) || !exact_sum(pj[c], pm[c])) flag = 1;
-                }
-            }
-            const int64_t at = 2 * ((int64_t)A + p);
-            rec64[at] = make_float4(__int_as_float(__double2loint(n[0])), __int_as_float(__double2hiint(n[0])),
-                                    __int_as_float(__double2loint(n[1])), __int_as_float(__double2hiint(n[1])));
-            rec64[at + 1] = make_float4(__int_as_float(__double2loint(n[2])), __int_as_float(__double2hiint(n[2])),
-                                        __int_as_float(w), __int_as_float(flag));
-        }
-    }
-}
-
-cudaError_t launch_build_rec64(const float4 *site, const float4 *rel, const float4 *cells, int64_t M, int64_t nrec,
-                               float4 *rec64, int sms, cudaStream_t s) {
-    if (M <= 0) return cudaSuccess;
-    (void)nrec;
-    const int blocks = (int)std::min<int64_t>((M + 127) / 128, (int64_t)sms * 16);
-    build_rec64_kernel<<<blocks, 128, 0, s>>>(site, rel, cells, M, rec64);
     count_launches(1);
     return cudaGetLastError();
 }

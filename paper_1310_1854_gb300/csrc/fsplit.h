@@ -61,6 +61,29 @@ VG_HD bool split_double_int(double x, float &hi, float &lo) {
     return true;
 }
 
+// x as float32, cut to its top 24 significant bits (error below 2^-23 |x|) with
+// integer operations; |x| < 2^-126 gives 0, and values beyond float32's range
+// (inf and NaN among them) are converted in float64.
+VG_HD float dtrunc(double x) {
+    const uint64_t t = dbits(x);
+    const uint32_t h = (uint32_t)(t >> 32);
+    const uint32_t e = (h >> 20) & 0x7ffu;
+    if (e - 897u > 253u) return e <= 896u ? 0.0f : (float)x;
+    return fbits((h & 0x80000000u) | (((h & 0x7fffffffu) - (896u << 20)) << 3) | ((uint32_t)t >> 29));
+}
+
+// (double)x with integer operations where x is normal
+VG_HD double fexact(float x) {
+    uint32_t b;
+    memcpy(&b, &x, 4);
+    const uint32_t a = b & 0x7fffffffu;
+    if (a - 0x00800000u >= 0x7f000000u) return (double)x;  // zero, subnormal, inf, NaN
+    const uint64_t t = ((uint64_t)((b & 0x80000000u) | ((a >> 3) + (896u << 20))) << 32) | (b << 29);
+    double d;
+    memcpy(&d, &t, 8);
+    return d;
+}
+
 // Order key of a float64 value: for non-NaN a, b, a <= b exactly when
 // dkey(a) <= dkey(b) as signed integers (-0 and +0 share a key).
 VG_HD int64_t dkey(double x) {

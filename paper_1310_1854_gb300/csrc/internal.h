@@ -51,12 +51,12 @@ void build_blocks(const double *box, const std::vector<double> &bbox, int64_t M,
 // stored in an array for batched launches. Cells are in the library's
 // internal (Morton) order.
 //
-// cells    absolute cell blocks (float64 form and rechecks), float4: cell i
+// cells    absolute cell blocks (float64 searches of a whole cell), float4: cell i
 //          starts at A_i with a header (bits of the caller's id, bits of the
 //          neighbour count c, rho, bits of F_i) followed by c records (x, y, z
 //          of the neighbour's site, bits of the neighbour's offset A_j, or of
 //          a wall id -1..-6).
-// rel      relative cell blocks (float32 form), float4: cell i starts at F_i
+// rel      relative cell blocks (float32 search), float4: cell i starts at F_i
 //          (even) with (x, y, z of p_i, bits of the record count c4) and
 //          (bits of the caller's id, rho, N1max, bits of A_i), followed by c4
 //          records: (fl(p_j - p_i) as float32, bits of F_j) for every cell
@@ -75,11 +75,6 @@ struct GridDev {
     const int32_t *perm;
     const int32_t *blk_off;
     const float4 *blk_rec;
-    // float64 form: per entry of `cells`, 32 bytes (two float4) holding the
-    // record's n = p_j - p_m as three doubles, its id (neighbour's offset in
-    // `cells`, or wall id) and a flag set where n or p_j + p_m is not exact
-    // in float64 (then the record is evaluated from its float coordinates)
-    const float4 *rec64;
     double lo[3], hi[3];      // domain box
     double bscale[3];         // blocks per unit length along each axis
     int64_t lokey[3], hikey[3];        // order keys of lo and hi (exact box test)
@@ -109,13 +104,24 @@ struct GridDev {
 // float64 set-up is cheap) and read once by the traversal kernel when the
 // ray starts (64 bytes).
 struct RayPrep {
-    int32_t cell;             // start cell: internal id (float64 form), offset of its relative
-                              // block (float32 form); -1 outside the box, -2 direction not unit
+    int32_t cell;             // offset of the start cell's relative block; -1 outside the box,
+                              // -2 direction not unit
     int32_t wall;             // wall the ray leaves through (Eq. 5), -1..-6
     float tmax_hi, tmax_lo;   // distance to that wall, as a float pair
     float r0_hi[3], r0_lo[3]; // origin as float pairs
     float k_hi[3], k_lo[3];   // direction as float pairs
 };
+
+// The same for the float64 form.
+struct RayPrep64 {
+    int32_t cell;             // as in RayPrep: offset of the start cell's relative block, or -1, -2
+    int32_t wall;             // the wall ahead, -1..-6 or -7 (sphere), where t_lo and t_hi name one
+    float t_lo, t_hi;         // bounds on the distance to the domain's boundary from the origin as the
+                              // float64 form evaluates it anywhere on the path; t_hi is infinite where
+                              // two walls are too close to call
+    double o[3], d[3];        // origin and direction
+};
+static_assert(sizeof(RayPrep) == 64 && sizeof(RayPrep64) == 64, "start records");
 
 // A batch work descriptor: rays of one grid.
 struct RaySetDev {

@@ -11,26 +11,31 @@
 // pairs, one 256-bit load each) and reduce the exit with shuffles.
 //
 // Cell blocks, in two forms; each crossing reads one contiguous block.
-//  * absolute (float64 form, rechecks): cell i owns a run of float4 at A_i:
-//    a header (caller's id, neighbour count, rho, F_i) and one record per
-//    neighbour (x, y, z of the neighbour's site, and its offset A_j, or a
-//    wall id -1..-6); the winner's record holds the next site and block.
-//  * relative (float32 form): cell i owns a run at F_i: (x, y, z of p_i,
-//    record count), (caller's id, rho, N1max, A_i), then one record per cell
-//    neighbour (n~ = fl(p_j - p_i), the neighbour's offset F_j), padded with
-//    NaN records to an even count of at least four. Walls are not records
-//    there: the wall ahead is one candidate from the ray's start record.
+//  * relative (the search of every form): cell i owns a run at F_i: (x, y, z of
+//    p_i, record count), (caller's id, rho, N1max, A_i), then one record per cell
+//    neighbour, nearest first (n~ = fl(p_j - p_i), the neighbour's offset F_j),
+//    padded with NaN records to an even count of at least four. Walls are not
+//    records there: the wall ahead is one candidate from the ray's start record.
+//  * absolute (float64 searches of a whole cell): cell i owns a run of float4 at
+//    A_i: a header (caller's id, neighbour count, rho, F_i) and one record per
+//    neighbour (x, y, z of the neighbour's site, and its offset A_j, or a wall id
+//    -1..-6).
 //
-// Two arithmetic forms of the exit search (Sect. 2.2, steps 1-3, Eq. 1-5):
-//  * float64: Eq. 4 and Eq. 5 evaluated as written, in the same operation
-//    order as a plain C implementation with contraction disabled, the
-//    current point updated as r <- r + s k.
-//  * float32 with recheck: each plane test runs in float32 in the frame of
-//    the current site, together with a rigorous bound on its rounding error.
-//    The exit is accepted when the upper bound of the winner lies below the
-//    lower bound of every other candidate; otherwise that one crossing is
-//    recomputed with the float64 form. The ray parameter t is kept as an
-//    unevaluated float pair, so no float64 work is needed per crossing.
+// The exit search (Sect. 2.2, steps 1-3, Eq. 1-5): each plane test runs in
+// float32 in the frame of the current site, together with a rigorous bound on
+// its rounding error. The exit is accepted when the upper bound of the winner
+// lies below the lower bound of every other candidate; otherwise that one
+// crossing is searched in float64. The forms differ in what they do with it:
+//  * float64: Eq. 4 or Eq. 5 for the accepted exit (or, where the bounds do not
+//    separate, for every candidate) as written, in the same operation order as
+//    a plain C implementation with contraction disabled, the current point
+//    updated as r <- r + s k. On the 10^5-site disk one crossing in about 10^4 is
+//    searched in float64. The float64 pipe bounds the form: testing every plane
+//    that may face ahead in float64 took 17.0 ms per 10^6 rays there, 3.46 ms
+//    now (about 50 float64 instructions per crossing instead of some 300).
+//  * float32: the length is the float32 quotient (or, with exact lengths, a
+//    float-pair one); the ray parameter t is kept as an unevaluated float pair,
+//    so no float64 work is needed per crossing.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -277,131 +282,54 @@ __device__ __forceinline__ bool wall64(const GridDev *gp, int w, const double *r
     return true;
 }
 
-// One record: bisector of the current site and the record's site (Eq. 1-4),
-// or a wall (Eq. 5), as the fraction num / den (num >= 0, den > 0). Returns
-// false if it is not a candidate (n.k <= 0).
+// The bisector of the current site and q's (Eq. 1-4) as the fraction num / den;
+// num is clamped at 0. INT: the site's coordinates widened with integer
+// operations (the float64 form's own step, bound by the float64 pipe).
+template <bool INT>
+__device__ __forceinline__ void fraction64(float4 q, double pmx, double pmy, double pmz, const double *r,
+                                           const double *k, double &num, double &den) {
+    const double px = INT ? fexact(q.x) : (double)q.x, py = INT ? fexact(q.y) : (double)q.y,
+                 pz = INT ? fexact(q.z) : (double)q.z;
+    const double nx = __dsub_rn(px, pmx), ny = __dsub_rn(py, pmy), nz = __dsub_rn(pz, pmz);
+    den = __dadd_rn(__dadd_rn(__dmul_rn(nx, k[0]), __dmul_rn(ny, k[1])), __dmul_rn(nz, k[2]));
+    // halving is exact for sums of float32 values, so the fused operation gives
+    // the same rounded difference of the midpoint and r
+    const double wx = INT ? __fma_rn(0.5, __dadd_rn(px, pmx), -r[0]) : __dsub_rn(__dmul_rn(__dadd_rn(px, pmx), 0.5), r[0]);
+    const double wy = INT ? __fma_rn(0.5, __dadd_rn(py, pmy), -r[1]) : __dsub_rn(__dmul_rn(__dadd_rn(py, pmy), 0.5), r[1]);
+    const double wz = INT ? __fma_rn(0.5, __dadd_rn(pz, pmz), -r[2]) : __dsub_rn(__dmul_rn(__dadd_rn(pz, pmz), 0.5), r[2]);
+    num = __dadd_rn(__dadd_rn(__dmul_rn(nx, wx), __dmul_rn(ny, wy)), __dmul_rn(nz, wz));
+    if ((int64_t)dbits(num) < 0) num = 0.0;  // negative, or -0
+}
+
+// One record: a bisector, or a wall (Eq. 5), as the fraction num / den (num
+// >= 0, den > 0). Returns false if it is not a candidate (n.k <= 0).
 __device__ __forceinline__ bool plane64(const GridDev *gp, float4 q, double pmx, double pmy, double pmz,
                                         const double *r, const double *k, double &num, double &den) {
     const int w = rec_w(q);
-    if (w >= 0) {
-        const double px = (double)q.x, py = (double)q.y, pz = (double)q.z;
-        const double nx = __dsub_rn(px, pmx), ny = __dsub_rn(py, pmy), nz = __dsub_rn(pz, pmz);
-        den = __dadd_rn(__dadd_rn(__dmul_rn(nx, k[0]), __dmul_rn(ny, k[1])), __dmul_rn(nz, k[2]));
-        if (!(den > 0.0)) return false;
-        const double wx = __dsub_rn(__dmul_rn(__dadd_rn(px, pmx), 0.5), r[0]);
-        const double wy = __dsub_rn(__dmul_rn(__dadd_rn(py, pmy), 0.5), r[1]);
-        const double wz = __dsub_rn(__dmul_rn(__dadd_rn(pz, pmz), 0.5), r[2]);
-        num = __dadd_rn(__dadd_rn(__dmul_rn(nx, wx), __dmul_rn(ny, wy)), __dmul_rn(nz, wz));
-        if (num < 0.0) num = 0.0;
-        return true;
-    }
-    return wall64(gp, w, r, k, num, den);
-}
-
-// float64 form, one record of the table of exact differences (see
-// GridDev::rec64): the same num and den as plane64 on the float record, with
-// fewer float64 operations. n = p_j - p_m is stored, and fma(0.5, n, p_m)
-// is (p_j + p_m) / 2 exactly, the value plane64 gets by rounding the sum and
-// halving it, because the table holds only records whose sum and difference
-// are exact; the flagged others go through plane64.
-__device__ __forceinline__ bool plane64x(const GridDev *gp, const float4 *crec, float4 xa, float4 xb, double pmx,
-                                         double pmy, double pmz, const double *r, const double *k, double &num,
-                                         double &den) {
-    const int w = __float_as_int(xb.z);
     if (w < 0) return wall64(gp, w, r, k, num, den);
-    if (__float_as_int(xb.w) != 0) return plane64(gp, __ldg(crec), pmx, pmy, pmz, r, k, num, den);
-    const double nx = __hiloint2double(__float_as_int(xa.y), __float_as_int(xa.x));
-    const double ny = __hiloint2double(__float_as_int(xa.w), __float_as_int(xa.z));
-    const double nz = __hiloint2double(__float_as_int(xb.y), __float_as_int(xb.x));
-    den = __dadd_rn(__dadd_rn(__dmul_rn(nx, k[0]), __dmul_rn(ny, k[1])), __dmul_rn(nz, k[2]));
-    if (!(den > 0.0)) return false;
-    const double wx = __dsub_rn(__fma_rn(0.5, nx, pmx), r[0]);
-    const double wy = __dsub_rn(__fma_rn(0.5, ny, pmy), r[1]);
-    const double wz = __dsub_rn(__fma_rn(0.5, nz, pmz), r[2]);
-    num = __dadd_rn(__dadd_rn(__dmul_rn(nx, wx), __dmul_rn(ny, wy)), __dmul_rn(nz, wz));
-    if (num < 0.0) num = 0.0;
-    return true;
+    fraction64<false>(q, pmx, pmy, pmz, r, k, num, den);
+    return den > 0.0;
 }
 
 // Exit of the cell whose records are blk[1..cnt] for the group: the
 // lexicographically smallest (s, id); returns the winner's record position
 // (1-based), kSphereWin if the exit is a spherical domain's boundary, or 0 if
-// there is no candidate, and its s in bs.
-// The float64 form's pre-test: false only for a record whose plane
-// certainly faces away (n.k <= 0), so that the float64 test can skip it; the
-// results are the same bits. The stored n's high words are truncated to
-// float32 with integer operations only (21 significant bits, relative error
-// below 2^-20; components below 2^-126 become 0) and dotted with k in
-// float32. The error against the exact n.k is at most ||n~||_1 (2^-20 +
-// 4.1 2^-24) + 3 2^-126; the bound b below is more than three times that,
-// so d <= -b leaves n.k < 0 by a margin far above float64's rounding. Walls
-// and flagged records always pass.
-__device__ __forceinline__ float hi_to_float(int h) {
-    const int e = (h >> 20) & 0x7ff;
-    const int bits = (h & (int)0x80000000) | ((e - 896) << 23) | ((h & 0xfffff) << 3);
-    return e > 896 ? __int_as_float(bits) : 0.0f;
-}
-
-__device__ __forceinline__ bool may_face64(float4 xa, float4 xb, const float *kf) {
-    if (__float_as_int(xb.z) < 0 || __float_as_int(xb.w) != 0) return true;
-    const float nx = hi_to_float(__float_as_int(xa.y));
-    const float ny = hi_to_float(__float_as_int(xa.w));
-    const float nz = hi_to_float(__float_as_int(xb.y));
-    const float d = __fmaf_rn(nz, kf[2], __fmaf_rn(ny, kf[1], __fmul_rn(nx, kf[0])));
-    const float b = __fmaf_rn(__fadd_rn(__fadd_rn(fabsf(nx), fabsf(ny)), fabsf(nz)), 0x1p-18f, 0x1p-120f);
-    return d > -b;
-}
-
-// FRAC (the float64 form) reads the records from x64, the block's entries
-// of the table of exact differences (two float4 per entry), and blk only for
-// flagged records; otherwise it reads the float records of blk.
+// there is no candidate, and its s in bs. Both forms come here only where the
+// float32 bounds do not separate the nearest two exits.
 template <int LPR, bool FRAC>
-__device__ __forceinline__ int exit64(const Hot &h, const GridDev *gp, const float4 *blk, const float4 *x64, int cnt,
-                                      double pmx, double pmy, double pmz, const double *r, const double *k,
-                                      const float *kf, unsigned gmask, int gl, double &bs) {
+__device__ __forceinline__ int exit64(const Hot &h, const GridDev *gp, const float4 *blk, int cnt, double pmx,
+                                      double pmy, double pmz, const double *r, const double *k, unsigned gmask, int gl,
+                                      double &bs) {
     double bn = 0.0, bd = 1.0;
     int bp = 0, bw = 0;
-    if (FRAC) {
-        // A warp issues a float64 instruction for all its lanes if any needs
-        // it, so a lane first marks which of its records may face ahead
-        // (float32 pre-test, up to 32 at a time) and then runs the float64
-        // test over those alone: the warp's float64 work follows the lane
-        // with the most candidates, not the one with the most records.
-        for (int base = 1 + gl; base <= cnt; base += 32 * LPR) {
-            unsigned m = 0;
-            for (int i = 0; i < 32; i++) {
-                const int p = base + i * LPR;
-                if (p > cnt) break;
-                float4 xa, xb;
-                ldg_pair(x64 + 2 * p, xa, xb);  // 32-byte entries
-                if (may_face64(xa, xb, kf)) m |= 1u << i;
-            }
-            while (m) {
-                const int p = base + (__ffs(m) - 1) * LPR;
-                m &= m - 1;
-                float4 xa, xb;
-                ldg_pair(x64 + 2 * p, xa, xb);
-                double n, d;
-                if (plane64x(gp, blk + p, xa, xb, pmx, pmy, pmz, r, k, n, d)) {
-                    const int w = __float_as_int(xb.z);
-                    if (better64<true>(h, n, d, w, bn, bd, bw, bp != 0)) {
-                        bn = n;
-                        bd = d;
-                        bp = p;
-                        bw = w;
-                    }
-                }
-            }
-        }
-    }
-    // the float32 form's recheck: every record of blk, s divided out
-    for (int p = 1 + gl; !FRAC && p <= cnt; p += LPR) {
+    for (int p = 1 + gl; p <= cnt; p += LPR) {
         const float4 q = __ldg(blk + p);
         double n, d;
         if (plane64(gp, q, pmx, pmy, pmz, r, k, n, d)) {
-            n = __ddiv_rn(n, d);
-            if (better64<false>(h, n, d, rec_w(q), bn, bd, bw, bp != 0)) {
+            if (!FRAC) n = __ddiv_rn(n, d);
+            if (better64<FRAC>(h, n, d, rec_w(q), bn, bd, bw, bp != 0)) {
                 bn = n;
+                if (FRAC) bd = d;
                 bp = p;
                 bw = rec_w(q);
             }
@@ -500,8 +428,8 @@ static __device__ __noinline__ int locate64(const GridDev *gp, double x, double 
 // Nearest site (internal id), -1 outside the closed box. With fp32 the
 // squared distances are float32 and the winner is accepted when
 // D2 - E(D2) > D1 + E(D1), E(D) = u (10 D + 4 X sqrt D), X = max |x_c|,
-// which bounds the rounding error of a float32 squared distance; otherwise
-// the list is rescanned in float64. *rechecked is set when that happened.
+// which (with 2^-140 for sums in the subnormal range) bounds the rounding error
+// of a float32 squared distance; otherwise the list is rescanned in float64. *rechecked is set when that happened.
 // A block's list is ordered by the sites' distance from the block's centre
 // c, so the float32 scan can stop early: a site not scanned yet is at least
 // as far from c as the last one scanned, s, hence at least |s - c| - |p - c|
@@ -513,7 +441,7 @@ static __device__ __noinline__ int locate64(const GridDev *gp, double x, double 
 // records pad them; a NaN distance never wins), so they can be read in pairs
 // (PAIRS; the traversal kernel's rare relocation reads them one by one).
 template <bool PAIRS>
-static __device__ __noinline__ int locate_point(const GridDev *gp, const LocPt P, bool fp32, int *rechecked) {
+__device__ __forceinline__ int locate_point(const GridDev *gp, const LocPt P, bool fp32, int *rechecked) {
     if (!inside(gp, P)) return -1;
     int bi[3];
     const int b = block_of(gp, P, bi);
@@ -534,7 +462,8 @@ static __device__ __noinline__ int locate_point(const GridDev *gp, const LocPt P
             rp = __fsqrt_rn(__fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex))));
         }
         // |p - c| rounded up, plus p's low words: subtracted from the bound
-        const float slack = __fadd_ru(__fmul_ru(rp, 1.0f + 16.0f * kU), __fmul_ru(4.0f * kU, X));
+        // (2^-70: square roots of sums rounded in the subnormal range)
+        const float slack = __fadd_ru(__fmul_ru(rp, 1.0f + 16.0f * kU), __fmaf_ru(4.0f * kU, X, 0x1p-70f));
         for (int i = beg; i < end; i += 2) {
             float4 q[2];
             if (PAIRS) {
@@ -566,12 +495,17 @@ static __device__ __noinline__ int locate_point(const GridDev *gp, const LocPt P
         }
         if (i1 >= 0 && D2 == __int_as_float(0x7f800000)) return i1;  // a single candidate
         const float s1 = sqrtf(D1), s2 = sqrtf(D2);
-        const float E1 = 1.0001f * kU * __fmaf_rn(10.0f, D1, 4.0f * X * s1);
-        const float E2 = 1.0001f * kU * __fmaf_rn(10.0f, D2, 4.0f * X * s2);
+        const float E1 = __fmaf_rn(1.0001f * kU, __fmaf_rn(10.0f, D1, 4.0f * X * s1), 0x1p-140f);
+        const float E2 = __fmaf_rn(1.0001f * kU, __fmaf_rn(10.0f, D2, 4.0f * X * s2), 0x1p-140f);
         if (i1 >= 0 && s2 > 8.0f * kU * X && __fsub_rd(D2, E2) > __fadd_ru(D1, E1)) return i1;
         if (rechecked) *rechecked = 1;
     }
     return locate64(gp, P.x[0], P.x[1], P.x[2], beg, end);
+}
+
+// out of line for the traversal kernels, which come here only after a nudge
+static __device__ __noinline__ int relocate_point(const GridDev *gp, const LocPt P, bool fp32) {
+    return locate_point<false>(gp, P, fp32, nullptr);
 }
 
 // ---------------------------------------------------------------------------
@@ -788,13 +722,13 @@ __device__ __forceinline__ int find_set(const RaySetDev *sets, int nsets, int64_
 // of that latency is hidden, so each instance is held to the largest count
 // that still gives it one more block of 128 threads per SM: 72 (seven
 // blocks) for tau, the adjoint and interaction sampling, 80 (six) for
-// segment lists (both forms) and the batch. The float64 tau traversal, bound
-// by the FP64 pipe, is left alone (80 registers; held to 72 it was slower).
+// segment lists and the batch. The float64 form, bound by the FP64 pipe, gets
+// 96 (five blocks; 80, 72 and 64 took 2, 4 and 7 % longer).
 // The per-ray values that a crossing of the float32 form reads once live in
 // shared memory, which is what lets the float32 instances fit.
 template <bool FP64, int MODE, bool BATCH, bool XL>
 constexpr int trace_max_regs() {
-    return FP64 ? (MODE == MODE_SEGS ? 80 : 255) : (BATCH || MODE == MODE_SEGS || XL) ? 80 : 72;
+    return FP64 ? 96 : (BATCH || MODE == MODE_SEGS || XL) ? 80 : 72;
 }
 
 // Ray queue. A warp takes up to 32 rays from the global counter at a time and
@@ -850,10 +784,11 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
     Hot h{a.g1.cells, a.g1.rel, a.g1.site};
     float kappa = a.g1.kappa;
     int max_steps = (int)min(a.g1.max_steps, (int64_t)0x7fffffff);
-    // float64 form: current point and direction (and the direction in
-    // float32 for the pre-test of the planes)
+    // float64 form: current point and direction, the distance gone in float32
+    // and the bounds on the boundary's distance (both only bound the wall)
     double r64[3] = {0, 0, 0}, k64[3] = {0, 0, 0};
-    float kf64[3] = {0.f, 0.f, 0.f};
+    float gone = 0.f, wlo = 0.f, whi = 0.f;
+    int wall = 0;
     // float32 form: origin and direction as float pairs, ray parameter t, wall
     // exit. Only the high words of the direction (used by every plane test)
     // and t stay in registers; the origin pairs, the low words of the
@@ -1060,23 +995,23 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 att = 1.f;
             }
             // the start record was prepared by the start-cell kernel
-            const RayPrep *pr = q_rec + slot;
-            int m;
+            const float4 *p4 = reinterpret_cast<const float4 *>(q_rec + slot);
+            const float4 a0 = p4[0];
+            const int m = __float_as_int(a0.x);
             if (FP64) {
-                m = pr->cell;
-                if (m >= 0) {
-                    const double *o = rs->origin + 3 * li;
-                    const double *d = rs->dir + 3 * li;
-                    for (int c = 0; c < 3; c++) {
-                        r64[c] = __ldg(o + c);
-                        k64[c] = __ldg(d + c);
-                        kf64[c] = __double2float_rn(k64[c]);
-                    }
+                wall = __float_as_int(a0.y);
+                wlo = a0.z;
+                whi = a0.w;
+                gone = 0.f;
+                const double *od = reinterpret_cast<const double *>(p4 + 1);
+                for (int c = 0; c < 3; c++) {
+                    r64[c] = od[c];
+                    k64[c] = od[3 + c];
+                    float lo;
+                    split_pair(k64[c], Kh[c], lo);  // K rounded to float32
                 }
             } else {
-                const float4 *p4 = reinterpret_cast<const float4 *>(pr);
-                const float4 a0 = p4[0], a1 = p4[1], a2 = p4[2], a3 = p4[3];
-                m = __float_as_int(a0.x);
+                const float4 a1 = p4[1], a2 = p4[2], a3 = p4[3];
                 tmh_ = a0.z;
                 tml_ = a0.w;
                 R0h_(0) = a1.x; R0h_(1) = a1.y; R0h_(2) = a1.z;
@@ -1085,17 +1020,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 Kl_(0) = a3.y;  Kl_(1) = a3.z;  Kl_(2) = a3.w;
             }
             status = m == -2 ? RAY_BAD_DIR : (m < 0 ? RAY_OUTSIDE : RAY_OK);
-            if (status == RAY_OK) {
-                if (FP64) {
-                    const float4 q = __ldg(&h.site[m]);
-                    pmx = q.x;
-                    pmy = q.y;
-                    pmz = q.z;
-                    B = rec_w(__ldg(h.rel + rec_w(q) + 1));  // absolute block of the cell
-                } else {
-                    B = m;  // relative block; the site comes with its header
-                }
-            }
+            if (status == RAY_OK) B = m;  // relative block; the site comes with its header
             if (status != RAY_OK) {
                 if (gl == 0) {
                     VG_STAT(status == RAY_OUTSIDE ? S_OUT : S_BAD);
@@ -1119,20 +1044,13 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
         if (ray < 0) continue;
 
         // ---------------- one exit decision ----------------
-        // float64 form: absolute block A (header: caller, count, rho, F);
-        // float32 form: relative block F (site and count, then caller, rho,
-        // N1max, A).
-        const float4 *blk = FP64 ? h.cells + B : h.rel + B;
+        // the cell's relative block: site and count, then caller, rho, N1max, A
+        const float4 *blk = h.rel + B;
         float4 hdr, hdr1;
-        if (FP64) {
-            hdr = __ldg(blk);
-            hdr1 = hdr;
-        } else {
-            ldg_pair(blk, hdr, hdr1);  // relative blocks start on 32-byte boundaries
-        }
-        const int cnt = FP64 ? hdr_count(hdr) : __float_as_int(hdr.w);
+        ldg_pair(blk, hdr, hdr1);  // relative blocks start on 32-byte boundaries
+        const int cnt = __float_as_int(hdr.w);
         const int caller = hdr_caller(hdr1);
-        const float rho = FP64 ? hdr.z : hdr1.y;
+        const float rho = hdr1.y;
         bool ended = false;
         double s64 = 0.0;      // float64 length (float64 form or recheck)
         bool from64 = FP64;
@@ -1140,21 +1058,8 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
         float len_lo = 0.f;    // exact lengths: the low word of the length
         bool found = false;    // an exit was found
         bool to_wall = false;  // ... and it is a wall
-        int nextB = 0;         // block offset of the next cell (same form as B)
-        float4 qn = make_float4(0.f, 0.f, 0.f, 0.f);  // float64 form: the winner's record
-        if (FP64) {
-            const int win = exit64<LPR, true>(h, gp, blk, a.g1.rec64 + 2 * (int64_t)B, cnt, (double)pmx, (double)pmy,
-                                              (double)pmz, r64, k64, kf64, gmask, gl, s64);
-            if (win == kSphereWin) {
-                found = true;
-                to_wall = true;
-            } else if (win > 0) {
-                qn = __ldg(blk + win);
-                found = true;
-                to_wall = rec_w(qn) < 0;
-                nextB = rec_w(qn);
-            }
-        } else {
+        int nextB = 0;         // relative block of the next cell
+        {
             const float4 *recs = blk + 1;  // records recs[1..cnt]
             float4 f0{}, f1{}, f2{}, f3{};
             if (LPR == 1) {
@@ -1164,29 +1069,52 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             pmx = hdr.x;
             pmy = hdr.y;
             pmz = hdr.z;
-            const float rx = local_coord(R0h_(0), R0l_(0), Kh[0], Kl_(0), th, tl, pmx);
-            const float ry = local_coord(R0h_(1), R0l_(1), Kh[1], Kl_(1), th, tl, pmy);
-            const float rz = local_coord(R0h_(2), R0l_(2), Kh[2], Kl_(2), th, tl, pmz);
+            // the current point in the frame of the site, to within 2u|r| + e_r
+            float rx, ry, rz;
+            if (FP64) {
+                rx = dtrunc(__dsub_rn(r64[0], fexact(pmx)));
+                ry = dtrunc(__dsub_rn(r64[1], fexact(pmy)));
+                rz = dtrunc(__dsub_rn(r64[2], fexact(pmz)));
+            } else {
+                rx = local_coord(R0h_(0), R0l_(0), Kh[0], Kl_(0), th, tl, pmx);
+                ry = local_coord(R0h_(1), R0l_(1), Kh[1], Kl_(1), th, tl, pmy);
+                rz = local_coord(R0h_(2), R0l_(2), Kh[2], Kl_(2), th, tl, pmz);
+            }
             const float r1 = __fadd_rn(__fadd_rn(fabsf(rx), fabsf(ry)), fabsf(rz));
             // the error terms of r and of the wall distance from t_max (no
             // shared-memory reads)
-            const float tmax_h = tmh_;
+            const float tmax_h = FP64 ? wlo : tmh_;
             const float scale = BATCH ? (float)gp->scale : (float)a.g1.scale;
-            const float rr = __fmaf_rn(kCB, r1, 2.0f * (16.0f * kU2 * (scale + tmax_h)));
+            // the float64 form's own rounding, 2^-29 of these terms, goes into
+            // them, and dtrunc's cut at 2^-126 into e_r
+            const float er = __fmaf_rn(16.0f * kU2, __fadd_rn(scale, tmax_h), FP64 ? 0x1p-124f : 0.0f);
+            const float rr = __fmaf_rn(FP64 ? 1.0001f * kCB : kCB, r1, 2.0f * er);
             const float n1m = hdr1.z;  // the cell's bound on |n|_1
             // the rounding bound of den~ plus 2^-126 (see consider32)
-            const float dden = __fadd_ru(__fmul_ru(kCDen, n1m), kDivMin);
-            const float dnum = __fmul_ru(n1m, __fmaf_ru(kCA, n1m, rr));
+            const float dden = __fadd_ru(__fmul_ru(FP64 ? 1.0001f * kCDen : kCDen, n1m), kDivMin);
+            const float dnum = __fmul_ru(n1m, __fmaf_ru(FP64 ? 1.0001f * kCA : kCA, n1m, rr));
             // the wall ahead is one more candidate: s_w = t_max - t
-            float sw, swl;
-            two_sum(tmh_, -th, sw, swl);
-            sw = __fadd_rn(sw, __fadd_rn(swl, __fsub_rn(tml_, tl)));
-            const float Ew = __fmaf_rn(3.0f * kU, fabsf(sw), 16.0f * kU2 * tmax_h);
-            const float lw = __fsub_rd(sw, Ew);
+            float sw, lw, uw;
+            if (FP64) {
+                // t is off by less than (steps + 2) 2u t (each length cut to
+                // 24 bits and added with one rounding)
+                const float Eg = __fmul_ru((float)(steps + 8) * (2.0f * kU), gone);
+                sw = 0.f;
+                lw = __fsub_rd(__fsub_rd(wlo, gone), Eg);
+                uw = steps < 32768 ? __fadd_ru(__fsub_ru(whi, gone), Eg) : __int_as_float(0x7f800000);
+                if (steps >= 32768) lw = 0.f;  // the bounds hold no longer: search in float64
+            } else {
+                float swl;
+                two_sum(tmh_, -th, sw, swl);
+                sw = __fadd_rn(sw, __fadd_rn(swl, __fsub_rn(tml_, tl)));
+                const float Ew = __fmaf_rn(3.0f * kU, fabsf(sw), 16.0f * kU2 * tmax_h);
+                lw = __fsub_rd(sw, Ew);
+                uw = __fadd_ru(sw, Ew);
+            }
             Stop32 e;
             e.rr = __fmaf_rn(rz, rz, __fmaf_rn(ry, ry, __fmul_rn(rx, rx)));
             e.rk2 = 2.0f * __fmaf_rn(rz, Kh[2], __fmaf_rn(ry, Kh[1], __fmul_rn(rx, Kh[0])));
-            const float er18 = 0x1p18f * (16.0f * kU2 * (scale + tmax_h));
+            const float er18 = 0x1p18f * er;
             e.rrm = fmaxf(e.rr, __fmul_rn(er18, er18));
             e.step = __fmul_rn(n1m, kStopStep);
             Cand32 c;
@@ -1206,7 +1134,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             Plane32 w1{0.f, 1.f, 0.f, 0.f};
             float4 qw = make_float4(0.f, 0.f, 0.f, 0.f);
             if (wall_wins) {
-                upper = __fadd_ru(sw, Ew);
+                upper = uw;
             } else if (LPR == 1 || c.p1 > 0) {
                 if (LPR == 1) {
                     w1 = Plane32{c.num1, c.den1, dnum, dden};  // kept by the exit search
@@ -1233,7 +1161,33 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                                      Kh[2], f);
                 apart = f.w1 == c.w1 && upper < f.L2;
             }
-            if (apart) {
+            // the float64 form takes any scale: where products of the cell's
+            // differences would leave float32's normal range it searches itself
+            if (FP64) apart = apart && n1m > 0x1p-50f && n1m < 0x1p60f;
+            if (apart && FP64) {
+                // the exit is known: Eq. 4 (or Eq. 5, or the sphere) in float64
+                // for it alone, with the operations of a search of the cell
+                found = true;
+                double num = 0.0, den = 1.0;
+                if (!wall_wins) {
+                    nextB = rec_w(qw);
+                    const float4 q = __ldg(h.rel + nextB);  // the winner's site heads its block
+                    fraction64<true>(q, fexact(pmx), fexact(pmy), fexact(pmz), r64, k64, num, den);
+                } else {
+                    to_wall = true;
+                    if (wall == kSphereWall) {
+                        num = sphere_exit64(gp, r64, k64);
+                    } else {  // wall64's fraction for the wall the ray faces
+                        const int axis = (-wall - 1) >> 1;
+                        const double rc = axis == 0 ? r64[0] : axis == 1 ? r64[1] : r64[2];
+                        const double kc = axis == 0 ? k64[0] : axis == 1 ? k64[1] : k64[2];
+                        num = (wall & 1) ? __dsub_rn(rc, a.g1.lo[axis]) : __dsub_rn(a.g1.hi[axis], rc);
+                        if ((int64_t)dbits(num) < 0) num = 0.0;
+                        den = fabs(kc);
+                    }
+                }
+                s64 = __ddiv_rn(num, den);
+            } else if (apart) {
                 found = true;
                 if (wall_wins) {
                     len = fmaxf(sw, 0.0f);
@@ -1251,22 +1205,30 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                     nextB = rec_w(qw);
                 }
             } else {
-                // float64 recheck of this crossing from r = r0 + t k, on the
-                // absolute block of the cell
-                if (gl == 0) VG_STAT(S_RE);
-                const RaySetDev *rs = BATCH ? &a.sets[set] : &a.s1;
-                const double *o = rs->origin + 3 * li;
-                const double *d = rs->dir + 3 * li;
+                // float64 search of the cell's absolute block: the float64
+                // form's own search, or the float32 form's recheck from r = r0
+                // + t k
+                if (!FP64 && gl == 0) VG_STAT(S_RE);
                 double kd[3], rp[3];
-                const double t = __dadd_rn((double)th, (double)tl);
-                for (int cc = 0; cc < 3; cc++) {
-                    kd[cc] = __ldg(d + cc);
-                    rp[cc] = __fma_rn(t, kd[cc], __ldg(o + cc));
+                if (FP64) {
+                    for (int cc = 0; cc < 3; cc++) {
+                        kd[cc] = k64[cc];
+                        rp[cc] = r64[cc];
+                    }
+                } else {
+                    const RaySetDev *rs = BATCH ? &a.sets[set] : &a.s1;
+                    const double *o = rs->origin + 3 * li;
+                    const double *d = rs->dir + 3 * li;
+                    const double t = __dadd_rn((double)th, (double)tl);
+                    for (int cc = 0; cc < 3; cc++) {
+                        kd[cc] = __ldg(d + cc);
+                        rp[cc] = __fma_rn(t, kd[cc], __ldg(o + cc));
+                    }
                 }
                 const float4 *ablk = h.cells + rec_w(hdr1);
                 const int acnt = hdr_count(__ldg(ablk));
-                const int win = exit64<LPR, false>(h, gp, ablk, nullptr, acnt, (double)pmx, (double)pmy, (double)pmz,
-                                                   rp, kd, nullptr, gmask, gl, s64);
+                const int win = exit64<LPR, FP64>(h, gp, ablk, acnt, (double)pmx, (double)pmy, (double)pmz, rp, kd, gmask,
+                                                  gl, s64);
                 if (win == kSphereWin) {
                     found = true;
                     to_wall = true;
@@ -1276,7 +1238,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                     to_wall = rec_w(qa) < 0;
                     if (!to_wall) nextB = rec_w(__ldg(h.cells + rec_w(qa)));  // F of the next cell
                 }
-                len = __double2float_rn(s64);
+                if (!FP64) len = __double2float_rn(s64);
                 from64 = true;
             }
         }
@@ -1316,6 +1278,28 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             B = nextB;
             continue;
         }
+        if (FP64 && found) {
+            // tau and the point for every lane before the paths part (a step of
+            // zero length adds zero to both): the float64 pipe bounds this form,
+            // and the lanes whose ray ends would run these again on their own
+            tau64 = __dadd_rn(tau64, __dmul_rn(__dmul_rn(fexact(kappa), fexact(rho)), s64));
+            for (int c = 0; c < 3; c++) r64[c] = __dadd_rn(r64[c], __dmul_rn(s64, k64[c]));
+            gone = __fadd_rn(gone, dtrunc(s64));
+        }
+        if (FP64 && found && !to_wall && (int64_t)dbits(s64) > 0 && steps + 1 < max_steps) {
+            // the same for the float64 form
+            if (MODE == MODE_SEGS && gl == 0) {
+                pend = true;
+                pend_cell = caller;
+                pend_ray = (int)ray;
+                pend_len = (SegLen)s64;
+            }
+            steps++;
+            nseg++;
+            zrun = 0;
+            B = nextB;
+            continue;
+        }
         bool interacted = false;  // interaction mode: the package interacts in this cell
 
         steps++;
@@ -1324,7 +1308,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             relocate = true;  // no exit found (Sect. 2.2): nudge over epsilon and locate again
             if (gl == 0) VG_STAT(S_NOEXIT);
         } else {
-            const bool positive = FP64 ? (s64 > 0.0) : (len > 0.0f);
+            const bool positive = FP64 ? (int64_t)dbits(s64) > 0 : len > 0.0f;
             if (positive) {
                 if (MODE == MODE_SEGS && gl == 0) {
                     pend = true;  // stored at the top of the next iteration
@@ -1356,9 +1340,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                     }
                 }
                 nseg++;
-                if (FP64) {
-                    tau64 = __dadd_rn(tau64, __dmul_rn(__dmul_rn((double)kappa, (double)rho), s64));
-                } else {
+                if (!FP64) {
                     // Kahan-compensated sum of kappa rho l
                     const float y = __fsub_rn(__fmul_rn(__fmul_rn(kappa, rho), len), tauc);
                     const float tt = __fadd_rn(tau32, y);
@@ -1373,7 +1355,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             if (MODE == MODE_INTERACT && interacted) to_wall = true;  // the path ends here
             // advance the point
             if (FP64) {
-                for (int c = 0; c < 3; c++) r64[c] = __dadd_rn(r64[c], __dmul_rn(s64, k64[c]));
+                // done above
             } else if (from64) {
                 ff_add_double(th, tl, s64);
             } else if (XL) {
@@ -1384,11 +1366,6 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             if (to_wall) {
                 ended = true;
             } else {
-                if (FP64) {  // the float32 form reads the site from the next block
-                    pmx = qn.x;
-                    pmy = qn.y;
-                    pmz = qn.z;
-                }
                 B = nextB;
                 // more zero-length steps in a row than the grid allows: nudge
                 relocate = zrun > 0 && zrun > (BATCH ? gp->zmax : a.g1.zmax);
@@ -1400,6 +1377,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             double x[3];
             if (FP64) {
                 for (int c = 0; c < 3; c++) r64[c] = __dadd_rn(r64[c], __dmul_rn(gp->eps64, k64[c]));
+                gone = __fadd_rn(gone, (float)gp->eps64);
                 for (int c = 0; c < 3; c++) x[c] = r64[c];
             } else {
                 ff_add_double(th, tl, gp->eps32);
@@ -1407,16 +1385,11 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 const double t = __dadd_rn((double)th, (double)tl);
                 for (int c = 0; c < 3; c++) x[c] = __fma_rn(t, __ldg(rs->dir + 3 * li + c), __ldg(rs->origin + 3 * li + c));
             }
-            const int nm = locate_point<false>(gp, loc_point(x[0], x[1], x[2]), !FP64, nullptr);
+            const int nm = relocate_point(gp, loc_point(x[0], x[1], x[2]), !FP64);
             if (nm < 0) {
                 ended = true;
             } else {
-                const float4 q = __ldg(&h.site[nm]);
-                pmx = q.x;
-                pmy = q.y;
-                pmz = q.z;
-                B = rec_w(q);
-                if (FP64) B = rec_w(__ldg(h.rel + B + 1));  // absolute block of the cell
+                B = rec_w(__ldg(&h.site[nm]));
             }
         }
         if (!ended && steps >= max_steps) {

@@ -1,14 +1,16 @@
-"""The traversal loop's ray queue and early stop of the exit search (GPU).
+"""The traversal loop's ray queue, early stop and float32 search (GPU).
 
 The queue hands a warp up to 32 rays at a time and the search leaves out the
 records that lie too far from the site: neither may change a result, so every
-comparison is exact (bit for bit).
+comparison is exact (bit for bit). The float64 form searches in float32 with
+error bounds and evaluates the exit in float64: its paths are the oracle's.
 """
 import numpy as np
 import pytest
 import torch
 
 import gen
+import oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +90,52 @@ def test_early_stop_takes_the_same_paths(kind):
     c = vg.trace(O, D, precision="fp64", segments=True)
     if kind != "lattice":        # rays through edges may order ties otherwise
         assert torch.equal(a.seg_off, c.seg_off) and torch.equal(a.seg_cell, c.seg_cell)
+
+
+@pytest.mark.parametrize("sphere", [None, tuple(gen.UNIT_BALL)])
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -70, 2.0 ** 40])
+def test_float64_form_at_the_boundary(scale, sphere):
+    """Rays along the walls, off them by nothing to 1e-3, with direction
+    components down to 1e-300, and rays that graze the sphere: the domain's
+    exit is where the float32 bounds are widest. Segment lengths to 1e-12 as
+    the other float64 tests."""
+    from paper_1310_1854_gb300 import VoronoiGrid
+    g = gen.make_ball_grid(800, 45) if sphere else gen.make_uniform_grid(800, 45)
+    rng = gen.rng_for(46)
+    n = 6000
+    rays = (gen.ball_rays if sphere else gen.uniform_rays)(n, 47)
+    o, d = rays.origin, rays.dir
+    ax, side = rng.integers(0, 3, n), rng.choice([-1.0, 1.0], n)
+    i = np.arange(n)
+    if sphere is None:
+        o[i, ax] = side * (1.0 - rng.choice([0.0, 1e-16, 1e-12, 1e-9, 1e-6, 1e-3], n))
+        d[i, ax] = side * rng.choice([0.0, 1e-300, 1e-40, 1e-17, 1e-9, 1e-5, 1e-2], n) * rng.choice([-1.0, 1.0], n)
+        d[i, (ax + 1) % 3] += 0.25  # not zero
+        d /= np.linalg.norm(d, axis=1, keepdims=True)
+    else:
+        u = gen.isotropic_dirs(n, rng)
+        t = np.cross(u, gen.isotropic_dirs(n, rng))
+        t /= np.linalg.norm(t, axis=1, keepdims=True)
+        o[:] = u * (1.0 - rng.choice([1e-12, 1e-9, 1e-6, 1e-3], n))[:, None]
+        d[:] = t + side[:, None] * rng.choice([0.0, 1e-9, 1e-5, 1e-2], n)[:, None] * u
+        d /= np.linalg.norm(d, axis=1, keepdims=True)
+    S, box = g.sites * scale, g.box * scale
+    sp = None if sphere is None else tuple(np.array(sphere) * scale)
+    o = np.ascontiguousarray(o * scale)
+    off, idx = oracle.csr(oracle.cells(S, box), len(S))
+    ref = oracle.trace(S, box, g.rho.astype(np.float64), o, d, off=off, idx=idx, **({"sphere": sp} if sp else {}))
+    ok = np.nonzero(ref.near_tie == 0)[0]
+    assert ok.size > 0.5 * n
+    vg = VoronoiGrid(S, box, sphere=sp)
+    vg.set_density(dev(g.rho))
+    for lanes in (1, 4):
+        vg.set_launch(fp64_lanes_per_ray=lanes)
+        r = vg.trace(dev(o), dev(d), precision="fp64", segments=True)
+        so, sc, sl = r.seg_off.cpu().numpy(), r.seg_cell.cpu().numpy(), r.seg_len.cpu().numpy()
+        diag = np.linalg.norm(box[3:] - box[:3])
+        for k in ok:
+            rc, rl = ref.segments(k)
+            assert np.array_equal(sc[so[k]:so[k + 1]], rc), k
+            gl = sl[so[k]:so[k + 1]]
+            assert np.all(np.abs(gl - rl) <= np.where(rl < 1e-6 * diag, 1e-12 * diag, 1e-12 * rl)), k
+        np.testing.assert_allclose(r.tau.cpu().numpy()[ok], ref.tau[ok], rtol=1e-12, atol=1e-300)
