@@ -562,6 +562,14 @@ __device__ __forceinline__ Plane32 plane32(float4 q, float rx, float ry, float r
 // sign shortcut of Sect. 2.2) would only add divergence; a masked result
 // costs nothing more. Positions past the count (several lanes per ray) are
 // masked by `valid`.
+// 1 / b to one ulp (at most 2^-23 relative) in one instruction: a subnormal b
+// counts as 0 and gives +inf, a subnormal result is 0
+__device__ __forceinline__ float rcp_ftz(float b) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(b));
+    return r;
+}
+
 template <bool KEEP>
 __device__ __forceinline__ void consider32(int pos, bool valid, float4 q, float rx, float ry, float rz, float dnumK,
                                            float dden, float Kx, float Ky, float Kz, Cand32 &c) {
@@ -577,9 +585,9 @@ __device__ __forceinline__ void consider32(int pos, bool valid, float4 q, float 
         // a plane facing away too, whatever value it gets can only lower
         // L2 or win without an upper bound (den_lo < 0), which sends the
         // crossing to the float64 recheck
-        lower = __fdividef(num_lo, fmaxf(den_hi, 0.0f));
+        lower = __fmul_rn(num_lo, rcp_ftz(fmaxf(den_hi, 0.0f)));
     } else {
-        lower = __fdividef(num_lo, den_hi);
+        lower = __fmul_rn(num_lo, rcp_ftz(den_hi));
         lower = (valid && den_hi > kDivMin) ? lower : __int_as_float(0x7f800000);
     }
     const bool b = lower < c.L1;
