@@ -70,7 +70,10 @@ int dmalloc(T **p, size_t n, int64_t &total) {
     *p = nullptr;
     if (n == 0) n = 1;
     cudaError_t e = cudaMalloc((void **)p, n * sizeof(T));
-    if (e != cudaSuccess) return fail(VGRID_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // or the next launch's check would report it
+        return fail(VGRID_ERR_NOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    }
     total += (int64_t)(n * sizeof(T));
     return VGRID_OK;
 }

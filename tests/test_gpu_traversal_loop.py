@@ -139,3 +139,50 @@ def test_float64_form_at_the_boundary(scale, sphere):
             gl = sl[so[k]:so[k + 1]]
             assert np.all(np.abs(gl - rl) <= np.where(rl < 1e-6 * diag, 1e-12 * diag, 1e-12 * rl)), k
         np.testing.assert_allclose(r.tau.cpu().numpy()[ok], ref.tau[ok], rtol=1e-12, atol=1e-300)
+
+
+def test_segment_buffers_guessed_counted_and_short_of_memory(monkeypatch):
+    """The lists are the same whether the buffers are sized on the first
+    guess, on the last call, after a count, or after a guess that is too small
+    or does not fit in memory; a generous guess is not kept alive."""
+    import paper_1310_1854_gb300 as pkg
+    g = gen.make_disk_grid(3000, 48)
+    rays = gen.disk_rays(2000, 49)
+    O, D = dev(rays.origin), dev(rays.dir)
+
+    def grid():
+        vg = pkg.VoronoiGrid(g.sites, g.box)
+        vg.set_density(dev(g.rho))
+        return vg
+
+    def same(r, q):
+        assert torch.equal(r.seg_off, q.seg_off) and torch.equal(r.seg_cell, q.seg_cell)
+        assert torch.equal(r.seg_len, q.seg_len) and torch.equal(r.tau, q.tau)
+        total = int(r.seg_off[-1])
+        assert r.seg_cell.numel() == total == r.stats["crossings"]
+        assert r.seg_cell.untyped_storage().nbytes() <= 4 * (1.5 * total + 4096) + 512
+
+    vg = grid()
+    want = vg.trace(O, D, segments=True)          # first guess
+    same(vg.trace(O, D, segments=True), want)     # from the last call
+    vg._seg_per_ray = 0.01
+    same(vg.trace(O, D, segments=True), want)     # too small: traced again
+    monkeypatch.setattr(pkg, "_SEG_GUESS_MAX", 10)
+    same(grid().trace(O, D, segments=True), want)  # counted first
+    monkeypatch.undo()
+    empty, asked = torch.empty, []
+
+    def tight(*a, **k):
+        n = a[0] if isinstance(a[0], int) else 0
+        if n > want.seg_cell.numel() and k.get("dtype") == torch.int32:
+            asked.append(n)
+            raise torch.cuda.OutOfMemoryError("CUDA out of memory (test)")
+        return empty(*a, **k)
+
+    monkeypatch.setattr(torch, "empty", tight)
+    r = grid().trace(O, D, segments=True)         # the guess does not fit
+    monkeypatch.undo()
+    assert asked
+    same(r, want)
+    none = vg.trace(O[:0], D[:0], segments=True)
+    assert none.seg_cell.numel() == 0 and int(none.seg_off[0]) == 0
