@@ -66,8 +66,7 @@ enum {
                                difference in float-pair arithmetic (within a
                                few u); float32 results as FP32_RECHECK's.
                                vgrid_trace, vgrid_trace_host and
-                               vgrid_trace_noalloc take it, with one lane per
-                               ray (the launch's lanes_per_ray is not used) */
+                               vgrid_trace_noalloc take it */
 };
 
 /* what vgrid_trace writes */
@@ -381,8 +380,11 @@ int vgrid_segments_grad(vgrid_t *g, const int64_t *seg_off, const int32_t *seg_c
 int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t N, const float *tau_int,
                    const float *weight, int32_t *cell, float *s, float *absorbed, vgrid_stream_t stream);
 
-/* Launch shape used by this grid's traversal kernels (NULL resets to the
- * built-in default). */
+/* Launch shape used by this grid's traversal kernels. NULL resets to the
+ * built-in default, which a new grid has: the shape that vgrid_get_launch
+ * returns, except that calls with too few rays to fill the GPU at one lane per
+ * ray use more lanes per ray (and smaller blocks in the float64 form). Results
+ * do not depend on the shape. */
 int vgrid_set_launch(vgrid_t *g, const vgrid_launch *launch);
 int vgrid_get_launch(const vgrid_t *g, vgrid_launch *launch);
 

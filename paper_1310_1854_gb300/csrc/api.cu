@@ -9,8 +9,11 @@
 #include <cmath>
 #include <cstring>
 #include <limits>
+#include <map>
 #include <memory>
+#include <mutex>
 #include <string>
+#include <tuple>
 #include <vector>
 
 #include "fsplit.h"
@@ -86,6 +89,7 @@ struct vgrid {
     int64_t M = 0;
     vgrid_opts opts{};
     vgrid_launch launch{1, 128, 0, 1, 0};
+    bool launch_auto = true;         // no shape was set: lanes per ray follow the number of rays
     GridDev hd{};
     GridDev *d_desc = nullptr;
     float4 *d_site = nullptr;
@@ -749,6 +753,7 @@ int vgrid_set_launch(vgrid_t *g, const vgrid_launch *l) {
     if (!g) return fail(VGRID_ERR_ARG, "null grid");
     if (!l) {
         g->launch = vgrid_launch{1, 128, 0, 1, 0};
+        g->launch_auto = true;
         return VGRID_OK;
     }
     if (!valid_lpr(l->lanes_per_ray)) return fail(VGRID_ERR_ARG, "lanes_per_ray must be 1, 2, 4 or 8");
@@ -758,6 +763,7 @@ int vgrid_set_launch(vgrid_t *g, const vgrid_launch *l) {
     if (l->blocks_per_sm < 0) return fail(VGRID_ERR_ARG, "blocks_per_sm must be >= 0");
     if (l->order < -1 || l->order > 1) return fail(VGRID_ERR_ARG, "order must be -1, 0 or 1");
     g->launch = *l;
+    g->launch_auto = false;
     return VGRID_OK;
 }
 
@@ -894,17 +900,69 @@ int ensure_chunks(vgrid_t *g, int64_t N, int64_t chunks, int slot_bytes) {
     return VGRID_OK;
 }
 
+// resident blocks per SM of a kernel at a block size, asked of the runtime once
+// per device
+int blocks_per_sm(const vg::TraceFn &fn, int block) {
+    static std::mutex mu;
+    static std::map<std::tuple<int, const void *, int>, int> known;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    int &n = known[{dev, fn.fn, block}];
+    if (n == 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn.fn, block, fn.smem(block)) != cudaSuccess || n < 1)) {
+        cudaGetLastError();
+        n = 0;
+        return 1;
+    }
+    return n;
+}
+
 // persistent grid size for a trace kernel
 int persistent_blocks(const vg::TraceFn &fn, const vgrid_launch &l, int sms, int64_t work_items) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn.fn, l.block, fn.smem(l.block)) != cudaSuccess ||
-        per_sm < 1)
-        per_sm = 1;
+    int per_sm = blocks_per_sm(fn, l.block);
     if (l.blocks_per_sm > 0 && l.blocks_per_sm < per_sm) per_sm = l.blocks_per_sm;
     int64_t blocks = (int64_t)per_sm * sms;
     const int64_t need = (work_items * l.lanes_per_ray + l.block - 1) / l.block;
     if (need < blocks) blocks = need > 0 ? need : 1;
     return (int)blocks;
+}
+
+// the kernel table's row for a precision
+int precision_row(int precision) {
+    return precision == VGRID_FP64 ? 1 : precision == VGRID_FP32_EXACT ? 2 : 0;
+}
+
+// The launch shape of a call of N rays (lanes_per_ray resolved for the row).
+// Without a shape set by the caller the lanes per ray follow N: a launch whose
+// rays do not fill the lanes lasts as long as its longest ray, a chain of
+// dependent loads per crossing that several lanes shorten. R is the rays one
+// lane each keeps resident (136,192 for float32 tau). Per call, us, with
+// 1 / 2 / 4 / 8 lanes on 10^5 disk sites: 50,000 rays (0.37 R) 456 / 434 / 390 /
+// 340; 75,000 483 / 483 / 422 / 357; 10^5 540 / 519 / 441 / 381; 150,000 620 / 580
+// / 482 / 497; 200,000 653 / 596 / 519 / 711; 300,000 687 / 639 / 680 / 940. On
+// 2 10^5 uniform sites, whose rays are more alike: 75,000 344 / 344 / 293 / 353;
+// 10^5 394 / 364 / 348 / 451; 150,000 427 / 393 / 481 / 643; 300,000 500 / 646 / 876
+// / 1229. The float64 form repeats its float64 work in every lane, so it takes
+// more than one only for very few rays (10^4 rays on 1000 sites: 128 / 111 / 133 /
+// 172) and where one lane each would leave a short second wave (10^5 on the disk:
+// 1630 / 1324), and single-warp blocks while they do not fill the SMs (the
+// float64 pipes of all SMs then share the rays evenly: 60,000 rays 1.28 -> 1.17
+// ms).
+vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N) {
+    vgrid_launch L = g->launch;
+    if (!g->launch_auto) {
+        if (row == 1 && L.fp64_lanes_per_ray) L.lanes_per_ray = L.fp64_lanes_per_ray;
+        return L;
+    }
+    L.lanes_per_ray = 1;
+    const double R = (double)persistent_blocks(kernels(1).get(row, mode), L, g->sms, INT64_MAX / 16) * L.block;
+    if (row == 1) {
+        L.lanes_per_ray = N <= 0.04 * R ? 8 : N <= 0.15 * R || (N > R && N <= 1.25 * R) ? 2 : 1;
+        if (N * L.lanes_per_ray < R) L.block = 32;
+    } else {
+        L.lanes_per_ray = N <= 0.5 * R ? 8 : N <= 0.95 * R ? 4 : N <= 2.0 * R ? 2 : 1;
+    }
+    return L;
 }
 
 int launch_trace(const vg::TraceFn &fn, const vgrid_launch &l, int sms, int64_t total, vg::TraceArgs &a, cudaStream_t s) {
@@ -943,29 +1001,15 @@ int locate_start(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l, int64
     return VGRID_OK;
 }
 
-// the kernel table's row for a precision (float32, float64, float32 with
-// exact lengths) and the launch shape it runs with
-static int precision_row(int precision, vgrid_launch &L) {
-    if (precision == VGRID_FP64) {
-        if (L.fp64_lanes_per_ray) L.lanes_per_ray = L.fp64_lanes_per_ray;
-        return 1;
-    }
-    if (precision == VGRID_FP32_EXACT) {
-        L.lanes_per_ray = 1;
-        return 2;
-    }
-    return 0;
-}
-
 // tau (and status) of n device-resident rays on s; the counters restart
 // only if reset_stats
 int trace_tau_chunk(vgrid_t *g, const double *origin, const double *dir, int64_t n, int precision, void *tau,
                     int32_t *status, bool reset_stats, cudaStream_t s) {
     int rc = ensure_start(g, n);
     if (rc) return rc;
-    vgrid_launch L = g->launch;
     const int fp64 = precision == VGRID_FP64;
-    const int row = precision_row(precision, L);
+    const int row = precision_row(precision);
+    const vgrid_launch L = shape_for(g, row, vg::MODE_TAU, n);
     const vg::KernelSet &ks = kernels(L.lanes_per_ray);
     RaySetDev set{origin, dir, tau, status, g->d_start, n, 0, 0, 0};
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, reset_stats ? g->d_stats : nullptr, s));
@@ -997,9 +1041,9 @@ int trace_tau_chunk(vgrid_t *g, const double *origin, const double *dir, int64_t
 // that read them take trace_tau_chunk instead).
 int trace_chunk_slot(vgrid_t *g, int k, const double *origin, const double *dir, int64_t n, int precision, void *tau,
                      int32_t *status, cudaStream_t s) {
-    vgrid_launch L = g->launch;
     const int fp64 = precision == VGRID_FP64;
-    const int row = precision_row(precision, L);
+    const int row = precision_row(precision);
+    const vgrid_launch L = shape_for(g, row, vg::MODE_TAU, n);
     const vg::TraceFn fn = kernels(L.lanes_per_ray).get(row, vg::MODE_TAU);
     cudaStream_t t = g->s_loc;
     VG_CUDA(cudaStreamWaitEvent(t, g->ev_in[k], 0));
@@ -1103,8 +1147,8 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
         origin = g->d_entry;
     }
     const int fp64 = precision == VGRID_FP64;
-    vgrid_launch L = g->launch;
-    const int row = precision_row(precision, L);
+    const int row = precision_row(precision);
+    const vgrid_launch L = shape_for(g, row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS, N);
     const vg::KernelSet &ks = kernels(L.lanes_per_ray);
     RaySetDev set{origin, dir, tau, ray_status, g->d_start, N, 0, 0, 0};
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
@@ -1321,7 +1365,9 @@ int vgrid_trace_grad(vgrid_t *g, const double *origin, const double *dir, int64_
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).get(0, vg::MODE_GRAD), g->launch, N, &order, s))) return rc;
+    const vgrid_launch L = shape_for(g, 0, vg::MODE_GRAD, N);
+    const vg::TraceFn fn = kernels(L.lanes_per_ray).get(0, vg::MODE_GRAD);
+    if ((rc = locate_start(g, fn, L, N, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
@@ -1336,7 +1382,7 @@ int vgrid_trace_grad(vgrid_t *g, const double *origin, const double *dir, int64_
     a.g1 = g->hd;
     a.s1 = set;
     mark(g, 1, 0, s);
-    rc = launch_trace(kernels(g->launch.lanes_per_ray).get(0, vg::MODE_GRAD), g->launch, g->sms, N, a, s);
+    rc = launch_trace(fn, L, g->sms, N, a, s);
     mark(g, 1, 1, s);
     return rc;
 }
@@ -1388,7 +1434,9 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, kernels(g->launch.lanes_per_ray).get(0, vg::MODE_INTERACT), g->launch, N, &order, s))) return rc;
+    const vgrid_launch L = shape_for(g, 0, vg::MODE_INTERACT, N);
+    const vg::TraceFn fn = kernels(L.lanes_per_ray).get(0, vg::MODE_INTERACT);
+    if ((rc = locate_start(g, fn, L, N, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
@@ -1406,7 +1454,7 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
     a.g1 = g->hd;
     a.s1 = set;
     mark(g, 1, 0, s);
-    rc = launch_trace(kernels(g->launch.lanes_per_ray).get(0, vg::MODE_INTERACT), g->launch, g->sms, N, a, s);
+    rc = launch_trace(fn, L, g->sms, N, a, s);
     mark(g, 1, 1, s);
     return rc;
 }
@@ -1596,11 +1644,15 @@ int grid_view(const struct vgrid *g, GridView *out) {
     out->sms = g->sms;
     out->d_desc = g->d_desc;
     out->hd = g->hd;
-    out->lanes_per_ray = g->launch.lanes_per_ray;
-    out->fp64_lanes_per_ray = g->launch.fp64_lanes_per_ray ? g->launch.fp64_lanes_per_ray : g->launch.lanes_per_ray;
-    out->block = g->launch.block;
-    out->blocks_per_sm = g->launch.blocks_per_sm;
     return 0;
+}
+
+TraceFn pick_trace(const struct vgrid *g, int row, int64_t N, int *block, int *blocks) {
+    const vgrid_launch L = shape_for(g, row, MODE_TAU, N);
+    const TraceFn fn = kernels(L.lanes_per_ray).get(row, MODE_TAU);
+    *block = L.block;
+    *blocks = persistent_blocks(fn, L, g->sms, N);
+    return fn;
 }
 
 }  // namespace vg

@@ -74,12 +74,16 @@ struct TraceFn {
 // (nullptr if absent); batch: the float32 tau kernel over many grids
 struct KernelSet {
     // fn[0]: float32 form, fn[1]: float64 form, fn[2]: float32 form with
-    // exact lengths (one lane per ray only)
+    // exact lengths
     const void *fn[3][NUM_MODES];
     const void *batch;
     TraceFn get(int row, int mode) const { return {fn[row][mode], trace_warp_bytes(row == 1, mode, false)}; }
     TraceFn get_batch() const { return {batch, trace_warp_bytes(false, MODE_TAU, true)}; }
 };
+
+// the tau kernel and launch shape of a call of N rays on g (api.cu), with g's
+// device current
+TraceFn pick_trace(const struct ::vgrid *g, int row, int64_t N, int *block, int *blocks);
 
 void kernel_table_lpr1(KernelSet &k);
 void kernel_table_lpr2(KernelSet &k);

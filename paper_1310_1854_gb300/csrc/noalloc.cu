@@ -93,24 +93,8 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
             rc = fail(VGRID_ERR_CUDA, cudaGetErrorString(e));
             break;
         }
-        if (fp64) v.lanes_per_ray = v.fp64_lanes_per_ray;
-        if (precision == VGRID_FP32_EXACT) v.lanes_per_ray = 1;  // its kernels take one lane per ray
-        vg::KernelSet ks{};
-        switch (v.lanes_per_ray) {
-            case 1: vg::kernel_table_lpr1(ks); break;
-            case 2: vg::kernel_table_lpr2(ks); break;
-            case 8: vg::kernel_table_lpr8(ks); break;
-            default: vg::kernel_table_lpr4(ks); break;
-        }
-        const vg::TraceFn fn = ks.get(precision == VGRID_FP32_EXACT ? 2 : fp64, vg::MODE_TAU);
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn.fn, v.block, fn.smem(v.block)) != cudaSuccess ||
-            per_sm < 1)
-            per_sm = 1;
-        if (v.blocks_per_sm > 0 && v.blocks_per_sm < per_sm) per_sm = v.blocks_per_sm;
-        int64_t blocks = (int64_t)per_sm * v.sms;
-        const int64_t need = (N * v.lanes_per_ray + v.block - 1) / v.block;
-        if (need < blocks) blocks = need;
+        int block = 0, blocks = 0;
+        const vg::TraceFn fn = vg::pick_trace(g, precision == VGRID_FP32_EXACT ? 2 : fp64, N, &block, &blocks);
         vg::TraceArgs a{};
         a.grids = v.d_desc;
         a.sets = dset;
@@ -121,7 +105,7 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
         a.g1 = v.hd;
         a.s1 = set;
         void *args[] = {&a};
-        e = cudaLaunchKernel(fn.fn, dim3((unsigned)blocks), dim3(v.block), args, fn.smem(v.block), s);
+        e = cudaLaunchKernel(fn.fn, dim3((unsigned)blocks), dim3(block), args, fn.smem(block), s);
         if (e != cudaSuccess) rc = fail(VGRID_ERR_CUDA, std::string("cudaLaunchKernel: ") + cudaGetErrorString(e));
     } while (0);
     if (prev != v.device) cudaSetDevice(prev);

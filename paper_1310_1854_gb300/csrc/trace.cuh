@@ -760,12 +760,12 @@ __device__ __forceinline__ void copy16_async(void *smem, const void *gmem) {
 }
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// XL: the float32 form with exact lengths (one lane per ray): decisions as
+// XL: the float32 form with exact lengths: decisions as
 // in the float32 form, each crossing's length from exact_length.
 template <int LPR, bool FP64, int MODE, bool BATCH, bool XL = false>
 __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, BATCH, XL>())) trace_kernel(TraceArgs a) {
     static_assert(LPR == 1 || LPR == 2 || LPR == 4 || LPR == 8, "lanes per ray");
-    static_assert(!XL || (LPR == 1 && !FP64 && !BATCH), "exact lengths: float32 form, one lane per ray");
+    static_assert(!XL || (!FP64 && !BATCH), "exact lengths: float32 form of one grid");
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LPR - 1);
     const int gbase = lane & ~(LPR - 1);

@@ -186,3 +186,33 @@ def test_segment_buffers_guessed_counted_and_short_of_memory(monkeypatch):
     same(r, want)
     none = vg.trace(O[:0], D[:0], segments=True)
     assert none.seg_cell.numel() == 0 and int(none.seg_off[0]) == 0
+
+
+@pytest.mark.parametrize("n", [100, 4_000, 20_000, 100_000, 130_000, 260_000])
+def test_default_shape_follows_the_rays(n):
+    """Without a shape set, few rays get several lanes each: the results are
+    those of one lane per ray, in every form and mode."""
+    from paper_1310_1854_gb300 import VoronoiGrid
+    g = gen.make_disk_grid(1500, 50)
+    rays = gen.disk_rays(n, 51)
+    O, D = dev(rays.origin), dev(rays.dir)
+    tint = torch.rand(n, device="cuda")
+
+    def everything(vg):
+        out = [vg.trace(O, D, precision=p).tau for p in ("fp32", "fp32_exact", "fp64")]
+        for p in ("fp32", "fp32_exact", "fp64"):
+            r = vg.trace(O, D, precision=p, segments=True, status=True)
+            out += [r.tau, r.seg_off, r.seg_cell, r.seg_len, r.status]
+        cell, s, _ = vg.interact(O, D, tint)
+        return out + [cell, s, vg.trace_host(O.cpu(), D.cpu()).tau.cuda()], vg.trace_grad(O, D, tint)
+
+    auto = VoronoiGrid(g.sites, g.box)
+    one = VoronoiGrid(g.sites, g.box)
+    one.set_launch(lanes_per_ray=1)
+    for vg in (auto, one):
+        vg.set_density(dev(g.rho))
+    (a, ga), (b, gb) = everything(auto), everything(one)
+    for i, (x, y) in enumerate(zip(a, b)):
+        assert torch.equal(x, y), i
+    # float32 atomics in another order: the same terms, some hundred per cell
+    torch.testing.assert_close(ga, gb, rtol=1e-4, atol=1e-6 * float(gb.abs().max()))
