@@ -149,6 +149,7 @@ struct vgrid {
     int64_t device_bytes = 0;
     int64_t host_fallback_cells = 0;
     int64_t rel_bytes = 0;           // bytes of the relative cell blocks
+    int64_t block_entries = 0;       // entries of all block lists
     // optional event record: {locate start, locate end} or {trace start, trace end}
     bool timing = false;
     std::vector<std::array<cudaEvent_t, 2>> ev_loc, ev_trace;
@@ -362,163 +363,26 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         return fail(o.gpu_build ? VGRID_ERR_CUDA : VGRID_ERR_BUILD, err);
     }
     lap(2, t_lap);
-    vg::build_blocks(bbox, g->cells.bbox, M, o.blocks_per_site, g->blocks, o.threads);
-    lap(3, t_lap);
-    if ((int64_t)(g->blocks.idx.size() + g->blocks.off.size()) + 2 >= ((int64_t)1 << 31)) {  // with the padding
-        delete g;
-        return fail(VGRID_ERR_NOMEM, "block lists exceed 2^31 entries; lower blocks_per_site");
-    }
-
-    // absolute cell blocks (offsets A): header (caller id, count, rho = 1,
-    // F), then one record per neighbour (site of the neighbour, its A) or
-    // wall. Relative cell blocks (offsets F, even): (site, record count),
-    // (caller id, rho = 1, N1max, A), then one record per cell neighbour
-    // (fl(p_j - p_i) in float32, its F), NaN-padded to an even count of
-    // records (at least four). N1max bounds |fl(p_j - p_i)|_1 over the
-    // records from above.
-    std::vector<int64_t> boffs(M + 1, 0), foffs(M + 1, 0);
-    std::vector<int32_t> ncell(M, 0);
-    vg::parallel_for(M, o.threads, 1 << 14, [&](int64_t b0, int64_t e0) {
-        for (int64_t i = b0; i < e0; i++)
-            for (int64_t q = g->cells.off[i]; q < g->cells.off[i + 1]; q++) ncell[i] += g->cells.idx[q] >= 0;
-    });
-    for (int64_t i = 0; i < M; i++) {
-        const int64_t b = g->cells.off[i], e = g->cells.off[i + 1];
-        boffs[i + 1] = boffs[i] + 1 + (e - b);
-        foffs[i + 1] = foffs[i] + 2 + std::max<int64_t>(4, (ncell[i] + 1) & ~(int64_t)1);
-    }
-    if (boffs[M] + 8 >= ((int64_t)1 << 31) || foffs[M] + 8 >= ((int64_t)1 << 31)) {
-        delete g;
-        return fail(VGRID_ERR_NOMEM, "cell blocks exceed 2^31 records");
-    }
-    const int64_t nrec = boffs[M] + 8;   // room past the end for the last block's reads
-    const int64_t nrel = foffs[M] + 8;
-    g->rel_bytes = nrel * (int64_t)sizeof(float4);
-    // every float of both block arrays is written below (in parallel), so
-    // they are allocated without the sequential zero fill
-    std::unique_ptr<float[]> blocks(new float[4 * nrec]), rel(new float[4 * nrel]);
-    std::vector<float> site4(4 * M);
-    auto put_int = [](float *dst, int32_t v) { std::memcpy(dst, &v, 4); };
-    const float fnan = std::numeric_limits<float>::quiet_NaN();
-    // every cell writes only its own blocks and site entry
-    vg::parallel_for(M, o.threads, 1 << 12, [&](int64_t i0, int64_t i1) {
-    std::vector<std::pair<double, int32_t>> near;  // cell neighbours by |p_j - p_i|^2
-    for (int64_t i = i0; i < i1; i++) {
-        const int64_t b = g->cells.off[i], e = g->cells.off[i + 1];
-        const float pi[3] = {(float)Si[3 * i + 0], (float)Si[3 * i + 1], (float)Si[3 * i + 2]};
-        float *h = &blocks[4 * boffs[i]];
-        put_int(h + 0, g->perm[i]);
-        put_int(h + 1, (int32_t)(e - b));
-        h[2] = 1.0f;
-        put_int(h + 3, (int32_t)foffs[i]);
-        float *f = &rel[4 * foffs[i]];
-        const int64_t c4 = foffs[i + 1] - foffs[i] - 2;
-        f[0] = pi[0];
-        f[1] = pi[1];
-        f[2] = pi[2];
-        put_int(f + 3, (int32_t)c4);
-        put_int(f + 4, g->perm[i]);
-        f[5] = 1.0f;
-        put_int(f + 7, (int32_t)boffs[i]);
-        double n1max = 0.0;
-        near.clear();
-        for (int64_t q = b; q < e; q++) {
-            float *r = &blocks[4 * (boffs[i] + 1 + (q - b))];
-            const int32_t j = g->cells.idx[q];
-            if (j >= 0) {
-                float pj[3];
-                for (int c = 0; c < 3; c++) pj[c] = (float)Si[3 * (int64_t)j + c];
-                r[0] = pj[0];
-                r[1] = pj[1];
-                r[2] = pj[2];
-                put_int(r + 3, (int32_t)boffs[j]);
-                double d2 = 0.0;
-                for (int c = 0; c < 3; c++) {
-                    volatile float d = pj[c] - pi[c];  // one float32 rounding, as on the device
-                    d2 += (double)d * (double)d;
-                }
-                near.emplace_back(d2, j);
-            } else {
-                r[0] = r[1] = r[2] = 0.0f;
-                put_int(r + 3, j);
-            }
+    // device buffers that the cell construction left, freed on every way out
+    struct CellsGuard {
+        vg::CellsOut &c;
+        ~CellsGuard() {
+            if (c.d_off) cudaFree(c.d_off);
+            if (c.d_idx) cudaFree(c.d_idx);
+            if (c.d_bbox) cudaFree(c.d_bbox);
+            c.d_off = nullptr;
+            c.d_idx = nullptr;
+            c.d_bbox = nullptr;
         }
-        // the relative records nearest neighbour first: the exit search stops
-        // once the rest lies too far from the site to be reached
-        std::sort(near.begin(), near.end());
-        int64_t k = 0;
-        for (; k < (int64_t)near.size(); k++) {
-            const int32_t j = near[(size_t)k].second;
-            float *rr = &f[4 * (2 + k)];
-            double n1 = 0.0;
-            for (int c = 0; c < 3; c++) {
-                volatile float d = (float)Si[3 * (int64_t)j + c] - pi[c];
-                rr[c] = d;
-                n1 += std::fabs((double)rr[c]);
-            }
-            put_int(rr + 3, (int32_t)foffs[j]);
-            n1max = std::max(n1max, n1);
-        }
-        for (; k < c4; k++) {
-            float *rr = &f[4 * (2 + k)];
-            rr[0] = rr[1] = rr[2] = fnan;
-            put_int(rr + 3, -8);
-        }
-        float n1f = (float)(n1max * (1.0 + 1e-6));
-        if ((double)n1f < n1max * (1.0 + 1e-6)) n1f = std::nextafter(n1f, INFINITY);
-        f[6] = n1f;
-        site4[4 * i + 0] = pi[0];
-        site4[4 * i + 1] = pi[1];
-        site4[4 * i + 2] = pi[2];
-        put_int(&site4[4 * i + 3], (int32_t)foffs[i]);
-    }
-    });
-    for (int64_t r = boffs[M]; r < nrec; r++) {
-        blocks[4 * r] = blocks[4 * r + 1] = blocks[4 * r + 2] = 0.0f;
-        put_int(&blocks[4 * r + 3], -8);
-    }
-    for (int64_t r = foffs[M]; r < nrel; r++) {
-        rel[4 * r] = rel[4 * r + 1] = rel[4 * r + 2] = fnan;
-        put_int(&rel[4 * r + 3], -8);
-    }
-    // block lists on the device: each padded to an even length with NaN
-    // records (id -1), so every list starts on a 32-byte boundary and is read
-    // in 256-bit pairs
-    const size_t nblk = g->blocks.off.size() - 1;
-    std::vector<int32_t> boff(nblk + 1, 0);
-    for (size_t i = 0; i < nblk; i++) {
-        const int64_t len = g->blocks.off[i + 1] - g->blocks.off[i];
-        boff[i + 1] = boff[i] + (int32_t)((len + 1) & ~(int64_t)1);
-    }
-
-    // coarse density grid for the ray order: about 2^18 near-cubic cells
-    // over the box, each holding (sites per unit volume)^(1/3), which is
-    // proportional to the cell faces a ray crosses per unit length
-    int32_t ddim[3];
-    {
-        const double ext[3] = {bbox[3] - bbox[0], bbox[4] - bbox[1], bbox[5] - bbox[2]};
-        const double cs = std::cbrt(ext[0] * ext[1] * ext[2] / 262144.0);
-        for (int c = 0; c < 3; c++) ddim[c] = (int32_t)std::min<long>(std::max<long>(std::lround(ext[c] / cs), 1), 256);
-    }
-    std::vector<float> dens((size_t)ddim[0] * ddim[1] * ddim[2], 0.0f);
-    {
-        std::vector<int64_t> cnt(dens.size(), 0);
-        for (int64_t i = 0; i < M; i++) {
-            int64_t idx = 0;
-            for (int c = 0; c < 3; c++) {
-                const double f = (Si[3 * i + c] - bbox[c]) / (bbox[3 + c] - bbox[c]) * ddim[c];
-                const int64_t ic = std::min<int64_t>(std::max<int64_t>((int64_t)f, 0), ddim[c] - 1);
-                idx = idx * ddim[c] + ic;
-            }
-            cnt[idx]++;
-        }
-        const double vol = (bbox[3] - bbox[0]) * (bbox[4] - bbox[1]) * (bbox[5] - bbox[2]) /
-                           ((double)ddim[0] * ddim[1] * ddim[2]);
-        for (size_t q = 0; q < dens.size(); q++) dens[q] = (float)std::cbrt(std::max(0.25, (double)cnt[q]) / vol);
-    }
-
-    lap(4, t_lap);
+    };
     if (o.host_only) {
+        vg::build_blocks(bbox, g->cells.bbox, M, o.blocks_per_site, g->blocks, o.threads);
+        lap(3, t_lap);
+        g->block_entries = (int64_t)g->blocks.idx.size();
+        if ((int64_t)(g->blocks.idx.size() + g->blocks.off.size()) + 2 >= ((int64_t)1 << 31)) {  // with the padding
+            delete g;
+            return fail(VGRID_ERR_NOMEM, "block lists exceed 2^31 entries; lower blocks_per_site");
+        }
         g->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         for (int c = 0; c < 3; c++) {
             g->hd.lo[c] = bbox[c];
@@ -535,89 +399,75 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     }
     g->device = dev;
     cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = cudaSuccess;
+    // The device arrays (cell blocks of both forms, block lists, coarse density
+    // grid), written by the device from the cells. Absolute cell blocks (offsets
+    // A): header (caller id, count, rho = 1, F), then one record per neighbour
+    // (site of the neighbour, its A) or wall. Relative cell blocks (offsets F,
+    // even): (site, record count), (caller id, rho = 1, N1max, A), then one
+    // record per cell neighbour (fl(p_j - p_i) in float32, its F), nearest first,
+    // NaN-padded to an even count of records (at least four). N1max bounds
+    // |fl(p_j - p_i)|_1 over the records from above. Block lists: ordered by the
+    // sites' distance from the block's centre, each padded to an even length
+    // with a NaN record (id -1), so that every list starts on a 32-byte boundary
+    // and is read in 256-bit pairs.
+    int32_t ddim[3];
+    {
+        // coarse density grid for the ray order: about 2^18 near-cubic cells
+        // over the box, each holding (sites per unit volume)^(1/3), which is
+        // proportional to the cell faces a ray crosses per unit length
+        const double ext[3] = {bbox[3] - bbox[0], bbox[4] - bbox[1], bbox[5] - bbox[2]};
+        const double cs = std::cbrt(ext[0] * ext[1] * ext[2] / 262144.0);
+        for (int c = 0; c < 3; c++) ddim[c] = (int32_t)std::min<long>(std::max<long>(std::lround(ext[c] / cs), 1), 256);
+    }
+    {
+        CellsGuard guard{g->cells};
+        std::vector<float4> site4(M);
+        vg::parallel_for(M, o.threads, 1 << 14, [&](int64_t i0, int64_t i1) {
+            for (int64_t i = i0; i < i1; i++)
+                site4[i] = make_float4((float)Si[3 * i], (float)Si[3 * i + 1], (float)Si[3 * i + 2], 0.0f);
+        });
+        vg::block_dims(bbox, M, o.blocks_per_site, g->blocks.dim);
+        vg::LayoutIn in{M, g->sms, bbox, {}, {}, site4.data(), g->perm.data(), g->cells.off.data(), g->cells.idx.data(),
+                        g->cells.bbox.data(), g->cells.d_off, g->cells.d_idx, g->cells.d_bbox};
+        for (int c = 0; c < 3; c++) {
+            in.bdim[c] = g->blocks.dim[c];
+            in.ddim[c] = ddim[c];
+        }
+        vg::LayoutOut lay{};
+        const int lrc = vg::build_layout(in, lay, err);
+        if (lrc != vg::LAYOUT_OK) {
+            free_grid(g);
+            return fail(lrc == vg::LAYOUT_NOMEM ? VGRID_ERR_NOMEM : VGRID_ERR_CUDA, err);
+        }
+        g->d_site = lay.site;
+        g->d_cells = lay.cells;
+        g->d_rel = lay.rel;
+        g->d_perm = lay.perm;
+        g->d_blk_off = lay.blk_off;
+        g->d_blk_rec = lay.blk_rec;
+        g->d_dens = lay.dens;
+        g->rel_bytes = lay.nrel * (int64_t)sizeof(float4);
+        g->block_entries = lay.entries;
+        const int64_t K = (int64_t)in.bdim[0] * in.bdim[1] * in.bdim[2];
+        g->device_bytes += (int64_t)sizeof(float4) * (M + lay.ncells + lay.nrel + lay.blk_records) +
+                           (int64_t)sizeof(int32_t) * (M + K + 1) +
+                           (int64_t)sizeof(float) * ddim[0] * ddim[1] * ddim[2];
+        g->phase_seconds[3] = lay.seconds[1];
+        g->phase_seconds[4] = lay.seconds[2];
+        g->phase_seconds[5] = lay.seconds[0];
+    }
     int rc = VGRID_OK;
 #define VG_ALLOC(p, n)                                              \
     if ((rc = dmalloc(&(p), (size_t)(n), g->device_bytes)) != 0) { \
         free_grid(g);                                               \
         return rc;                                                  \
     }
-    VG_ALLOC(g->d_site, M);
-    VG_ALLOC(g->d_cells, nrec);
-    VG_ALLOC(g->d_rel, nrel);
-    VG_ALLOC(g->d_perm, M);
-    VG_ALLOC(g->d_blk_off, boff.size());
-    VG_ALLOC(g->d_blk_rec, (size_t)boff[nblk] + 2);
-    VG_ALLOC(g->d_dens, dens.size());
     VG_ALLOC(g->d_desc, 1);
     VG_ALLOC(g->d_queue, 1);
     VG_ALLOC(g->d_stats, 1);
     VG_ALLOC(g->d_set, 1);
 #undef VG_ALLOC
-    cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_site, site4.data(), sizeof(float) * 4 * M, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_cells, blocks.get(), sizeof(float) * 4 * nrec, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_rel, rel.get(), sizeof(float) * 4 * nrel, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_perm, g->perm.data(), sizeof(int32_t) * M, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_blk_off, boff.data(), sizeof(int32_t) * boff.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(g->d_dens, dens.data(), sizeof(float) * dens.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-        const float fnan = std::numeric_limits<float>::quiet_NaN();
-        // every entry is written below (the lists in parallel, each with its
-        // NaN padding, then the two entries past the end), so the buffer is
-        // allocated without a fill
-        const size_t nbrec = (size_t)boff[nblk] + 2;
-        std::unique_ptr<float[]> brec(new float[4 * nbrec]);
-        auto put_nan = [&](size_t q) {
-            brec[4 * q + 0] = brec[4 * q + 1] = brec[4 * q + 2] = fnan;
-            put_int(&brec[4 * q + 3], -1);
-        };
-        put_nan(nbrec - 2);
-        put_nan(nbrec - 1);
-        // each list ordered by the sites' distance from its block's centre,
-        // flo_hi + (i + 1/2) fbw per axis in float32 (the operations the
-        // start-cell search repeats), ties by cell: the search stops once the
-        // rest of the list is certainly farther than its best site
-        const int32_t *bd = g->blocks.dim;
-        float fbw[3], flo[3];
-        for (int c = 0; c < 3; c++) {
-            fbw[c] = (float)((bbox[3 + c] - bbox[c]) / bd[c]);
-            flo[c] = (float)bbox[c];
-        }
-        vg::parallel_for((int64_t)nblk, o.threads, 1 << 12, [&](int64_t b0, int64_t b1) {
-            std::vector<std::pair<double, int32_t>> ord;
-            for (int64_t b = b0; b < b1; b++) {
-                const int64_t bk[3] = {b / ((int64_t)bd[1] * bd[2]), (b / bd[2]) % bd[1], b % bd[2]};
-                double cen[3];
-                for (int c = 0; c < 3; c++) {
-                    volatile float t = (float)bk[c] + 0.5f;
-                    volatile float m = t * fbw[c];
-                    cen[c] = (double)(float)(flo[c] + m);
-                }
-                ord.clear();
-                for (int64_t q = g->blocks.off[b]; q < g->blocks.off[b + 1]; q++) {
-                    const int32_t c = g->blocks.idx[q];
-                    double d2 = 0.0;
-                    for (int a = 0; a < 3; a++) {
-                        const double d = (double)(float)Si[3 * (int64_t)c + a] - cen[a];
-                        d2 += d * d;
-                    }
-                    ord.emplace_back(d2, c);
-                }
-                std::sort(ord.begin(), ord.end());
-                for (int64_t q = g->blocks.off[b]; q < g->blocks.off[b + 1]; q++) {
-                    const int32_t c = ord[(size_t)(q - g->blocks.off[b])].second;
-                    float *r = &brec[4 * ((size_t)boff[b] + (size_t)(q - g->blocks.off[b]))];
-                    r[0] = (float)Si[3 * (int64_t)c + 0];
-                    r[1] = (float)Si[3 * (int64_t)c + 1];
-                    r[2] = (float)Si[3 * (int64_t)c + 2];
-                    put_int(r + 3, c);
-                }
-                const size_t len = (size_t)(g->blocks.off[b + 1] - g->blocks.off[b]);
-                for (size_t q = (size_t)boff[b] + len; q < (size_t)boff[b + 1]; q++) put_nan(q);
-            }
-        });
-        e = cudaMemcpy(g->d_blk_rec, brec.get(), sizeof(float) * 4 * nbrec, cudaMemcpyHostToDevice);
-    }
 
     GridDev &hd = g->hd;
     hd.site = g->d_site;
@@ -633,7 +483,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         // on one part of the grid
         int l2 = 0;
         cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, g->device);
-        hd.ospatial = (double)nrel * sizeof(float4) > 0.5 * (double)l2 ? 16 : 1;
+        hd.ospatial = (double)g->rel_bytes > 0.5 * (double)l2 ? 16 : 1;
     }
     double dmax = 0;
     for (int c = 0; c < 3; c++) {
@@ -668,7 +518,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         free_grid(g);
         return fail(VGRID_ERR_CUDA, std::string("upload: ") + cudaGetErrorString(e));
     }
-    lap(5, t_lap);
     g->build_seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     *out = g;
     return VGRID_OK;
@@ -689,7 +538,7 @@ int vgrid_info(const vgrid_t *g, vgrid_info_t *info) {
     if (!g || !info) return fail(VGRID_ERR_ARG, "null argument");
     info->M = g->M;
     info->nnz = (int64_t)g->cells.idx.size();
-    info->block_entries = (int64_t)g->blocks.idx.size();
+    info->block_entries = g->block_entries;
     for (int c = 0; c < 3; c++) {
         info->block_dim[c] = g->blocks.dim[c];
         info->box[c] = g->hd.lo[c];

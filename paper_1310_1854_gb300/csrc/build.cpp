@@ -563,15 +563,20 @@ void morton_order(const double *S, int64_t M, const double *box, std::vector<int
 
 // Regular block grid over the box; each block lists the cells whose bounding
 // box overlaps it (Sect. 2.3).
+void block_dims(const double *box, int64_t M, double blocks_per_site, int32_t *dim) {
+    const double ext[3] = {box[3] - box[0], box[4] - box[1], box[5] - box[2]};
+    const double target = std::max(1.0, blocks_per_site * (double)M);
+    const double s = std::cbrt(ext[0] * ext[1] * ext[2] / target);
+    for (int c = 0; c < 3; c++)
+        dim[c] = (int32_t)std::min<long>(std::max<long>(std::lround(ext[c] / s), 1), 1024);
+}
+
+// The lists of a host-only grid (a device grid's are built on the device, by
+// the same rule: layout.cu)
 void build_blocks(const double *box, const std::vector<double> &bbox, int64_t M, double blocks_per_site,
                   BlocksOut &out, int threads) {
-    double ext[3] = {box[3] - box[0], box[4] - box[1], box[5] - box[2]};
-    double target = std::max(1.0, blocks_per_site * (double)M);
-    double s = std::cbrt(ext[0] * ext[1] * ext[2] / target);
-    for (int c = 0; c < 3; c++) {
-        long n = std::lround(ext[c] / s);
-        out.dim[c] = (int32_t)std::min<long>(std::max<long>(n, 1), 1024);
-    }
+    const double ext[3] = {box[3] - box[0], box[4] - box[1], box[5] - box[2]};
+    block_dims(box, M, blocks_per_site, out.dim);
     const int64_t K = (int64_t)out.dim[0] * out.dim[1] * out.dim[2];
     const double diag = std::sqrt(ext[0] * ext[0] + ext[1] * ext[1] + ext[2] * ext[2]);
     double maxabs = 0.0;

@@ -553,6 +553,8 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
             double tb[6];
             for (int c = 0; c < 6; c++) tb[c] = std::ldexp(box[c], k);
             const int rc = build_cells_gpu(T.data(), M, tb, threads, out, err, host_fallback_cells);
+            if (out.d_bbox) cudaFree(out.d_bbox);
+            out.d_bbox = nullptr;  // scaled
             for (double &v : out.vol) v = std::ldexp(v, -3 * k);
             for (double &v : out.bbox) v = std::ldexp(v, -k);
             return rc;
@@ -676,6 +678,12 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         count_launches(1);
         if ((e = cudaMemcpy(out.idx.data(), didx, sizeof(int) * out.off[M], cudaMemcpyDeviceToHost)) != cudaSuccess)
             return bad(e, "download");
+        out.d_off = doff;
+        out.d_idx = didx;
+        out.d_bbox = bbox;
+        doff = nullptr;
+        didx = nullptr;
+        bbox = nullptr;
         cleanup();
         return 0;
     }

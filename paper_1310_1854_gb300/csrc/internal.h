@@ -17,10 +17,15 @@ struct CellsOut {
     std::vector<int32_t> idx;   // neighbour ids (internal) and walls -1..-6
     std::vector<double> vol;    // cell volumes
     std::vector<double> bbox;   // 6 per cell
+    // device copies of off, idx and bbox where the GPU construction leaves
+    // them, for the caller to free; else NULL
+    int64_t *d_off = nullptr;
+    int32_t *d_idx = nullptr;
+    double *d_bbox = nullptr;
 };
 
 struct BlocksOut {
-    int32_t dim[3];
+    int32_t dim[3] = {1, 1, 1};
     std::vector<int64_t> off;   // K + 1
     std::vector<int32_t> idx;   // internal cell ids
 };
@@ -41,6 +46,8 @@ void morton_order(const double *sites, int64_t M, const double *box, std::vector
 // host threads (0: all cores); ranges of fewer than `grain` items stay on
 // one thread
 void parallel_for(int64_t n, int threads, int64_t grain, const std::function<void(int64_t, int64_t)> &fn);
+// blocks per axis of the block lists
+void block_dims(const double *box, int64_t M, double blocks_per_site, int32_t *dim);
 void build_blocks(const double *box, const std::vector<double> &bbox, int64_t M, double blocks_per_site,
                   BlocksOut &out, int threads = 0);
 

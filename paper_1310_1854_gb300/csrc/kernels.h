@@ -129,6 +129,34 @@ cudaError_t launch_locate(const GridDev *grids, const RaySetDev *sets, int nsets
                           int32_t *out_caller, int sms, cudaStream_t s);
 cudaError_t launch_permute_density(const float *rho_caller, const int32_t *perm, const float4 *site, int64_t M,
                                    float4 *cells, float4 *rel, cudaStream_t s);
+// Device arrays of a grid from its cells (layout.cu), on the current device.
+// site4, perm, off, idx, bbox: host, in the internal cell order; d_off, d_idx,
+// d_bbox: the same on the device where the cell construction left them
+// there, else NULL.
+struct LayoutIn {
+    int64_t M;
+    int sms;
+    const double *box;
+    int32_t bdim[3], ddim[3];   // block grid, coarse density grid
+    const float4 *site4;        // (x, y, z, -) per cell
+    const int32_t *perm;
+    const int64_t *off;
+    const int32_t *idx;
+    const double *bbox;
+    const int64_t *d_off;
+    const int32_t *d_idx;
+    const double *d_bbox;
+};
+struct LayoutOut {
+    float4 *site, *cells, *rel, *blk_rec;
+    int32_t *perm, *blk_off;
+    float *dens;
+    int64_t ncells, nrel, blk_records;  // float4 records of cells, rel, blk_rec
+    int64_t entries;                    // entries of all block lists, without padding
+    double seconds[3];                  // copies in, block lists, cell blocks
+};
+enum { LAYOUT_OK = 0, LAYOUT_NOMEM = 1, LAYOUT_CUDA = 2 };
+int build_layout(const LayoutIn &in, LayoutOut &out, std::string &err);
 // copy the segments of the chunks the traversal took (read from the chunk
 // cursor on the device, at most chunk_cap; see kSegChunk) of rays 0..N-1
 // into the CSR arrays at the scanned offsets off[0..N], unless off[N]
