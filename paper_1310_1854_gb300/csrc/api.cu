@@ -7,6 +7,7 @@
 #include <array>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <limits>
 #include <map>
@@ -120,7 +121,6 @@ struct vgrid {
     int64_t meta_cap = 0;
     int64_t *d_coff = nullptr;       // chunks per ray, scanned
     int64_t coff_cap = 0;
-    unsigned long long *d_cursor = nullptr;
     uint8_t *d_bin = nullptr;    // ray order: bins, counts, permutation
     uint32_t *d_hist = nullptr;
     int32_t *d_order = nullptr;
@@ -246,7 +246,7 @@ static void free_grid(vgrid_t *g) {
     if (g->d_hset) cudaFree(g->d_hset);
     void *ptrs[] = {g->d_desc,  g->d_site,  g->d_cells, g->d_rel,   g->d_dens,  g->d_bin,   g->d_hist,
                     g->d_order, g->d_perm,  g->d_blk_off, g->d_blk_rec, g->d_queue, g->d_stats, g->d_set,
-                    g->d_start, g->d_scan,  g->d_entry, g->d_slots, g->d_chunk_meta, g->d_chunk_inv, g->d_coff, g->d_cursor};
+                    g->d_start, g->d_scan,  g->d_entry, g->d_slots, g->d_chunk_meta, g->d_chunk_inv, g->d_coff};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete g;
@@ -693,7 +693,7 @@ int ensure_order(vgrid_t *g, int64_t N) {
 }
 
 int ensure_scan(vgrid_t *g, int64_t N) {
-    const int64_t need = vg::scan_tmp_elems(N);
+    const int64_t need = vg::segment_tmp_elems(N);
     if (need <= g->scan_cap) return VGRID_OK;
     if (g->d_scan) {
         cudaFree(g->d_scan);
@@ -711,10 +711,6 @@ int ensure_scan(vgrid_t *g, int64_t N) {
 // slot_bytes, their (ray, position) records and the inverse map, and the
 // chunk offsets of N rays
 int ensure_chunks(vgrid_t *g, int64_t N, int64_t chunks, int slot_bytes) {
-    if (!g->d_cursor) {
-        int rc = dmalloc(&g->d_cursor, 1, g->device_bytes);
-        if (rc) return rc;
-    }
     if (N + 1 > g->coff_cap) {
         if (g->d_coff) cudaFree(g->d_coff);
         g->device_bytes -= g->coff_cap * (int64_t)sizeof(int64_t);
@@ -1042,31 +1038,32 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     }
     if ((rc = ensure_scan(g, N))) return rc;
     if ((rc = ensure_chunks(g, N, chunks, fp64 ? 16 : 8))) return rc;
-    VG_CUDA(cudaMemsetAsync(g->d_cursor, 0, sizeof(unsigned long long), s));
+    // the chunk cursor sits with the counters, which the set-up kernel cleared
+    unsigned long long *const cursor = reinterpret_cast<unsigned long long *>(
+        reinterpret_cast<char *>(g->d_stats) + offsetof(StatsDev, cursor));
     a.seg_off = seg_off;
     a.seg_slots = g->d_slots;
     a.chunk_meta = g->d_chunk_meta;
-    a.chunk_cursor = g->d_cursor;
+    a.chunk_cursor = cursor;
     a.chunk_cap = chunks;
     mark(g, 1, 0, s);
     if ((rc = launch_trace(fn, L, g->sms, N, a, s))) return rc;
     mark(g, 1, 1, s);
-    VG_CUDA(vg::launch_exclusive_scan(seg_off, N, g->d_scan, s));
     // the copy compares the total with the capacity on the device, so the
-    // call synchronises once, at its end
+    // call synchronises once, at its end: one read of the counters, with the
+    // chunks taken; the crossings are the total (seg_off[N])
     const bool have = seg_cell && seg_len;
-    VG_CUDA(vg::launch_compact_segments(seg_off, N, chunks, g->d_cursor, g->d_chunk_meta, g->d_slots, fp64 != 0,
-                                        have ? seg_capacity : 0, g->d_coff, g->d_scan, g->d_chunk_inv, seg_cell,
-                                        seg_len, g->sms, s));
-    int64_t total = 0;
-    unsigned long long taken = 0;
-    VG_CUDA(cudaMemcpyAsync(&total, seg_off + N, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    VG_CUDA(cudaMemcpyAsync(&taken, g->d_cursor, sizeof(taken), cudaMemcpyDeviceToHost, s));
-    const int src = read_stats(g->d_stats, stats, s);  // synchronises
+    VG_CUDA(vg::launch_segment_lists(seg_off, N, chunks, cursor, g->d_chunk_meta, g->d_slots, fp64 != 0,
+                                     have ? seg_capacity : 0, g->d_coff, g->d_scan, g->d_chunk_inv, seg_cell, seg_len,
+                                     g->sms, s));
+    StatsDev h{};
+    const int src = read_stats(g->d_stats, stats, s, &h);  // synchronises
+    if (src == VGRID_ERR_CUDA) return src;
+    const int64_t total = (int64_t)h.crossings;
     if (total > seg_capacity || (total > 0 && !have))
         return fail(VGRID_ERR_CAPACITY, "segment buffers hold " + std::to_string(seg_capacity) + ", need " +
                                             std::to_string(total));
-    if ((int64_t)taken > chunks)  // cannot happen when the total fits (see above)
+    if ((int64_t)h.cursor > chunks)  // cannot happen when the total fits (see above)
         return fail(VGRID_ERR_CUDA, "segment chunk pool ran out");
     return src;
 }

@@ -452,19 +452,75 @@ __global__ void __launch_bounds__(kScanThreads) scan_fix_kernel(int64_t *data, i
         if (base + i < n) data[base + i] += add;
 }
 
-// Chunked segments -> CSR, in the order of the destination so that the
-// stores are coalesced: (1) chunks per ray, ceil(n / kSegChunk), scanned into
-// coff; (2) each used chunk c of ray r at position k is entered as
-// inv[coff[r] + k] = c; (3) kSegChunk threads per destination chunk copy its
-// slots to the ray's offset plus kSegChunk * k. The number of chunks the
-// traversal took and the total are read on the device: when the total
-// exceeds the caller's capacity (some chunks were never stored) steps 2 and
-// 3 do nothing, and only the offsets go back.
-__global__ void chunk_counts_kernel(const int64_t *off, int64_t N, int64_t *ccount) {
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < N; r += (int64_t)gridDim.x * blockDim.x)
-        ccount[r] = (__ldg(off + r + 1) - __ldg(off + r) + kSegChunk - 1) / kSegChunk;
+// Offsets of the rays' segments and of their chunks (ceil(n / kSegChunk)), both
+// scans in one pass over the counts: three kernels instead of seven, and the
+// counts are read once.
+__global__ void __launch_bounds__(kScanThreads) ray_scan_tiles_kernel(int64_t *off, int64_t n, int64_t *coff,
+                                                                     longlong2 *tile_sums) {
+    __shared__ int64_t ws[32];
+    const int64_t base = blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+    int64_t v[kScanItems], sum = 0, csum = 0;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+        v[i] = base + i < n ? off[base + i] : 0;
+        sum += v[i];
+        csum += (v[i] + kSegChunk - 1) / kSegChunk;
+    }
+    int64_t total, ctotal;
+    int64_t run = block_exclusive_scan(sum, ws, total), crun = block_exclusive_scan(csum, ws, ctotal);
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++) {
+        if (base + i < n) {
+            off[base + i] = run;
+            coff[base + i] = crun;
+        }
+        run += v[i];
+        crun += (v[i] + kSegChunk - 1) / kSegChunk;
+    }
+    if (threadIdx.x == 0) tile_sums[blockIdx.x] = make_longlong2(total, ctotal);
 }
 
+__global__ void __launch_bounds__(kScanThreads) ray_scan_sums_kernel(longlong2 *tile_sums, int64_t ntiles, int64_t *off_n,
+                                                                    int64_t *coff_n) {
+    __shared__ int64_t ws[32];
+    int64_t carry = 0, ccarry = 0;
+    for (int64_t b = 0; b < ntiles; b += kScanThreads) {
+        const int64_t i = b + threadIdx.x;
+        const longlong2 v = i < ntiles ? tile_sums[i] : make_longlong2(0, 0);
+        int64_t total, ctotal;
+        const int64_t ex = block_exclusive_scan(v.x, ws, total), cex = block_exclusive_scan(v.y, ws, ctotal);
+        if (i < ntiles) tile_sums[i] = make_longlong2(carry + ex, ccarry + cex);
+        carry += total;
+        ccarry += ctotal;
+    }
+    if (threadIdx.x == 0) {
+        *off_n = carry;
+        *coff_n = ccarry;
+    }
+}
+
+__global__ void __launch_bounds__(kScanThreads) ray_scan_fix_kernel(int64_t *off, int64_t n, int64_t *coff,
+                                                                   const longlong2 *tile_sums) {
+    const longlong2 add = tile_sums[blockIdx.x];
+    const int64_t base = blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+#pragma unroll
+    for (int i = 0; i < kScanItems; i++)
+        if (base + i < n) {
+            off[base + i] += add.x;
+            coff[base + i] += add.y;
+        }
+}
+
+// Chunked segments -> CSR, in the order of the destination so that the
+// stores are coalesced: each used chunk c of ray r at position k is entered as
+// inv[coff[r] + k] = c; then kSegChunk threads per destination chunk copy its
+// slots to the ray's offset plus kSegChunk * k. The number of chunks the
+// traversal took and the total are read on the device: when the total
+// exceeds the caller's capacity (some chunks were never stored) both do
+// nothing, and only the offsets go back. (Entering (c, r) in inv, so that a
+// chunk's slots and its ray's offsets load side by side, and two slots per
+// thread took 47 + 148 us for 28.7 10^6 segments instead of 36 + 133: the
+// inversion's scattered writes double and the copy's are 8 bytes apart.)
 __global__ void chunk_invert_kernel(const int2 *meta, const unsigned long long *cursor, int64_t chunk_cap,
                                     const int64_t *off, int64_t N, int64_t cap, const int64_t *coff, int32_t *inv) {
     if (__ldg(off + N) > cap) return;
@@ -506,17 +562,20 @@ static int grid_for(int64_t threads, int sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((threads + 255) / 256, (int64_t)sms * 8));
 }
 
-cudaError_t launch_compact_segments(const int64_t *off, int64_t N, int64_t chunk_cap, const unsigned long long *cursor,
-                                    const int2 *meta, const void *slots, bool fp64, int64_t cap, int64_t *coff,
-                                    int64_t *scan_tmp, int32_t *inv, int32_t *cell, void *len, int sms,
-                                    cudaStream_t s) {
-    if (N <= 0 || chunk_cap <= 0 || !cell || !len) return cudaSuccess;
-    chunk_counts_kernel<<<grid_for(N, sms), 256, 0, s>>>(off, N, coff);
-    count_launches(1);
-    cudaError_t e = launch_exclusive_scan(coff, N, scan_tmp, s);
-    if (e != cudaSuccess) return e;
+int64_t segment_tmp_elems(int64_t n) { return 2 * scan_tmp_elems(n); }
+
+cudaError_t launch_segment_lists(int64_t *off, int64_t N, int64_t chunk_cap, const unsigned long long *cursor,
+                                 const int2 *meta, const void *slots, bool fp64, int64_t cap, int64_t *coff,
+                                 int64_t *scan_tmp, int32_t *inv, int32_t *cell, void *len, int sms, cudaStream_t s) {
+    if (N <= 0) return cudaMemsetAsync(off, 0, sizeof(int64_t), s);
+    const int64_t tiles = (N + kScanTile - 1) / kScanTile;
+    longlong2 *const sums = reinterpret_cast<longlong2 *>(scan_tmp);
+    ray_scan_tiles_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(off, N, coff, sums);
+    ray_scan_sums_kernel<<<1, kScanThreads, 0, s>>>(sums, tiles, off + N, coff + N);
+    ray_scan_fix_kernel<<<(unsigned)tiles, kScanThreads, 0, s>>>(off, N, coff, sums);
+    count_launches(3);
+    if (chunk_cap <= 0 || !cell || !len) return cudaGetLastError();
     chunk_invert_kernel<<<grid_for(chunk_cap, sms), 256, 0, s>>>(meta, cursor, chunk_cap, off, N, cap, coff, inv);
-    count_launches(1);
     // destination chunks: coff[N] (read on the device), at most chunk_cap
     if (fp64)
         compact_segments_kernel<true><<<grid_for(chunk_cap * kSegChunk, sms), 256, 0, s>>>(off, coff, N, cap, inv,
@@ -524,7 +583,7 @@ cudaError_t launch_compact_segments(const int64_t *off, int64_t N, int64_t chunk
     else
         compact_segments_kernel<false><<<grid_for(chunk_cap * kSegChunk, sms), 256, 0, s>>>(off, coff, N, cap, inv,
                                                                                             meta, slots, cell, len);
-    count_launches(1);
+    count_launches(2);
     return cudaGetLastError();
 }
 

@@ -146,6 +146,7 @@ struct RaySetDev {
 // Counters accumulated on the device; mirrors vgrid_stats.
 struct StatsDev {
     unsigned long long rays, crossings, decisions, rechecks, fallbacks, zero_steps, step_limit, outside, bad_dir;
+    unsigned long long cursor;  // segment mode: chunks handed out, read back with the counters
 };
 
 

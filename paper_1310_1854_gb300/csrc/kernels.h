@@ -157,15 +157,17 @@ struct LayoutOut {
 };
 enum { LAYOUT_OK = 0, LAYOUT_NOMEM = 1, LAYOUT_CUDA = 2 };
 int build_layout(const LayoutIn &in, LayoutOut &out, std::string &err);
-// copy the segments of the chunks the traversal took (read from the chunk
-// cursor on the device, at most chunk_cap; see kSegChunk) of rays 0..N-1
-// into the CSR arrays at the scanned offsets off[0..N], unless off[N]
-// exceeds cap (then nothing is written); coff holds N+1 and inv chunk_cap
-// values of scratch, scan_tmp scan_tmp_elems(N)
-cudaError_t launch_compact_segments(const int64_t *off, int64_t N, int64_t chunk_cap, const unsigned long long *cursor,
-                                    const int2 *meta, const void *slots, bool fp64, int64_t cap, int64_t *coff,
-                                    int64_t *scan_tmp, int32_t *inv, int32_t *cell, void *len, int sms,
-                                    cudaStream_t s);
+// Segment lists in ray order. counts_to_off holds the segments per ray 0..N-1
+// and becomes their offsets off[0..N]; then the segments of the chunks the
+// traversal took (read from the chunk cursor on the device, at most
+// chunk_cap; see kSegChunk) are copied into the CSR arrays, unless off[N]
+// exceeds cap (then nothing is written) or chunk_cap is 0 or cell or len NULL.
+// coff holds N+1 and inv chunk_cap values of scratch, scan_tmp
+// segment_tmp_elems(N).
+int64_t segment_tmp_elems(int64_t n);
+cudaError_t launch_segment_lists(int64_t *counts_to_off, int64_t N, int64_t chunk_cap, const unsigned long long *cursor,
+                                 const int2 *meta, const void *slots, bool fp64, int64_t cap, int64_t *coff,
+                                 int64_t *scan_tmp, int32_t *inv, int32_t *cell, void *len, int sms, cudaStream_t s);
 // adjoint from segment lists: out[cell[k]] += g[r] * kappa * len[k] for the
 // segments k of every ray r (CSR offsets off[0..N])
 cudaError_t launch_segments_grad(const int64_t *off, const int32_t *cell, const float *len, int64_t N, const float *g,
