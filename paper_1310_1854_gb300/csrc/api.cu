@@ -787,13 +787,16 @@ int precision_row(int precision) {
 // / 482 / 497; 200,000 653 / 596 / 519 / 711; 300,000 687 / 639 / 680 / 940. On
 // 2 10^5 uniform sites, whose rays are more alike: 75,000 344 / 344 / 293 / 353;
 // 10^5 394 / 364 / 348 / 451; 150,000 427 / 393 / 481 / 643; 300,000 500 / 646 / 876
-// / 1229. The float64 form repeats its float64 work in every lane, so it takes
+// / 1229. Rays that enter from outside cross the whole domain and are more alike
+// still, so that throughput counts from fewer of them on: 10^4 into a ball of
+// 60,000 sites 228 / 188 / 153 / 138, 30,000 278 / 220 / 209 / 253, 50,000 294 / 262 /
+// 307 / 343, 75,000 315 / 330 / 364 / 476. The float64 form repeats its float64 work in every lane, so it takes
 // more than one only for very few rays (10^4 rays on 1000 sites: 128 / 111 / 133 /
 // 172) and where one lane each would leave a short second wave (10^5 on the disk:
 // 1630 / 1324), and single-warp blocks while they do not fill the SMs (the
 // float64 pipes of all SMs then share the rays evenly: 60,000 rays 1.28 -> 1.17
 // ms).
-vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N) {
+vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N, bool enter = false) {
     vgrid_launch L = g->launch;
     if (!g->launch_auto) {
         if (row == 1 && L.fp64_lanes_per_ray) L.lanes_per_ray = L.fp64_lanes_per_ray;
@@ -805,7 +808,8 @@ vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N) {
         L.lanes_per_ray = N <= 0.04 * R ? 8 : N <= 0.15 * R || (N > R && N <= 1.25 * R) ? 2 : 1;
         if (N * L.lanes_per_ray < R) L.block = 32;
     } else {
-        L.lanes_per_ray = N <= 0.5 * R ? 8 : N <= 0.95 * R ? 4 : N <= 2.0 * R ? 2 : 1;
+        const double f8 = enter ? 0.11 : 0.4, f4 = enter ? 0.27 : 0.75, f2 = enter ? 0.45 : 1.4;
+        L.lanes_per_ray = N <= f8 * R ? 8 : N <= f4 * R ? 4 : N <= f2 * R ? 2 : 1;
     }
     return L;
 }
@@ -993,7 +997,7 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     }
     const int fp64 = precision == VGRID_FP64;
     const int row = precision_row(precision);
-    const vgrid_launch L = shape_for(g, row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS, N);
+    const vgrid_launch L = shape_for(g, row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS, N, enter);
     const vg::KernelSet &ks = kernels(L.lanes_per_ray);
     RaySetDev set{origin, dir, tau, ray_status, g->d_start, N, 0, 0, 0};
     VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
