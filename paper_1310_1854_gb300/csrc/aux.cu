@@ -44,16 +44,18 @@ cudaError_t launch_prepare(RaySetDev *d_set, const RaySetDev &set, unsigned long
 // float32 (rechecked) or float64 distances;
 // PREP_FP32: float32 form (cell, direction check, wall exit of Eq. 5 and the
 // float pairs of origin and direction); PREP_FP64: float64 form (cell,
-// direction check, bounds on the wall exit, origin and direction). The caller's id of the cell goes to out_caller if given.
+// direction check, bounds on the wall exit, origin and direction). The caller's
+// id of the cell goes to out_caller if given.
 // One instance per kind of record, with the search inlined: the cells alone
 // then fit without spills.
 // Held to five blocks of 256 threads per SM (48 registers, a few spilled):
 // the kernel waits on its loads, and the extra warps hide more of that wait
-// than the spilled bytes cost.
+// than the spilled bytes cost. The cells alone need 40 registers: six blocks
+// (10^7 points of the 10^6-site disk 426 -> 405 us; seven spill, 430).
 template <int PREP>
-__global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets,
-                                                     int64_t total, int32_t *out_caller, uint8_t *bin,
-                                                     uint32_t *hist) {
+__global__ void __launch_bounds__(256, PREP == PREP_CELL32 || PREP == PREP_CELL64 ? 6 : 5)
+    locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int32_t *out_caller,
+                  uint8_t *bin, uint32_t *hist) {
     __shared__ uint32_t s_hist[kOrderBins];
     if (bin) {
         for (int b = threadIdx.x; b < kOrderBins; b += blockDim.x) s_hist[b] = 0u;
@@ -210,7 +212,10 @@ __global__ void __launch_bounds__(256, 5) locate_kernel(const GridDev *grids, co
 static cudaError_t launch_locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
                                         int32_t *out_caller, uint8_t *bin, uint32_t *hist, int sms, cudaStream_t s) {
     if (total <= 0) return cudaSuccess;
-    const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)sms * 16);
+    // many more blocks than fit: points differ in the records they scan, and the
+    // blocks that end early make room (8 / 16 / 32 / 64 per SM and one point per
+    // thread took 457 / 452 / 422 / 418 / 435 us for the same points)
+    const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)sms * 64);
     const dim3 g((unsigned)blocks);
     switch (prep) {
         case PREP_CELL32: locate_kernel<PREP_CELL32><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
