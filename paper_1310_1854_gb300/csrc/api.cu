@@ -106,7 +106,6 @@ struct vgrid {
     // work buffers
     unsigned long long *d_queue = nullptr;
     StatsDev *d_stats = nullptr;
-    RaySetDev *d_set = nullptr;
     RayPrep *d_start = nullptr;
     int64_t start_cap = 0;
     int64_t *d_scan = nullptr;
@@ -130,8 +129,7 @@ struct vgrid {
     double *d_hin[2] = {nullptr, nullptr};  // chunk origins then directions
     void *d_hout[2] = {nullptr, nullptr};   // chunk tau (8 bytes per ray)
     int32_t *d_hst[2] = {nullptr, nullptr}; // chunk status
-    // per slot also the start records, ray order, work counter and set
-    // descriptor, so that a chunk's start records can be prepared on s_loc
+    // per slot also the start records, ray order and work counter, so that a chunk's start records can be prepared on s_loc
     // while the previous chunk is traced (the start-cell pass then fills the
     // SMs that the traversal frees in its tail)
     RayPrep *d_hstart[2] = {nullptr, nullptr};
@@ -139,7 +137,6 @@ struct vgrid {
     int32_t *d_horder[2] = {nullptr, nullptr};
     uint32_t *d_hhist = nullptr;             // per slot 2 kOrderBins
     unsigned long long *d_hqueue = nullptr;  // per slot
-    RaySetDev *d_hset = nullptr;             // per slot
     int64_t host_cap = 0;
     int host_slot = 0;
     cudaStream_t s_h2d = nullptr, s_d2h = nullptr, s_loc = nullptr;
@@ -243,9 +240,8 @@ static void free_grid(vgrid_t *g) {
     if (g->s_loc) cudaStreamDestroy(g->s_loc);
     if (g->d_hhist) cudaFree(g->d_hhist);
     if (g->d_hqueue) cudaFree(g->d_hqueue);
-    if (g->d_hset) cudaFree(g->d_hset);
     void *ptrs[] = {g->d_desc,  g->d_site,  g->d_cells, g->d_rel,   g->d_dens,  g->d_bin,   g->d_hist,
-                    g->d_order, g->d_perm,  g->d_blk_off, g->d_blk_rec, g->d_queue, g->d_stats, g->d_set,
+                    g->d_order, g->d_perm,  g->d_blk_off, g->d_blk_rec, g->d_queue, g->d_stats,
                     g->d_start, g->d_scan,  g->d_entry, g->d_slots, g->d_chunk_meta, g->d_chunk_inv, g->d_coff};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -466,7 +462,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     VG_ALLOC(g->d_desc, 1);
     VG_ALLOC(g->d_queue, 1);
     VG_ALLOC(g->d_stats, 1);
-    VG_ALLOC(g->d_set, 1);
 #undef VG_ALLOC
 
     GridDev &hd = g->hd;
@@ -828,23 +823,27 @@ int64_t resident_lanes(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l)
     return (int64_t)persistent_blocks(fn, l, g->sms, INT64_MAX / 16) * l.block / l.lanes_per_ray;
 }
 
-// start records (float32 form, or float64 with fp64) for the set in
-// g->d_set; with the ray order (see vgrid_launch.order) also the
-// permutation, which goes to *order
-int locate_start(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l, int64_t N, const int32_t **order, cudaStream_t s,
-                bool fp64 = false) {
+// start records (float32 form, or float64 with fp64) for the rays of `set`; with
+// the ray order (see vgrid_launch.order) also the permutation, which goes to
+// *order. Clears g's work counter, and its counters with reset_stats.
+int locate_start(vgrid_t *g, const vg::TraceFn &fn, const vgrid_launch &l, const RaySetDev &set, const int32_t **order,
+                 cudaStream_t s, bool fp64 = false, bool reset_stats = true) {
     *order = nullptr;
+    const int64_t N = set.n;
     const int prep = fp64 ? vg::PREP_FP64 : vg::PREP_FP32;
+    vg::LocateArgs a{g->d_desc, nullptr, 1, set, N, nullptr, nullptr, nullptr, g->d_queue, reset_stats ? g->d_stats : nullptr};
     const bool want = l.order == 1 || (l.order == 0 && N >= 2 * resident_lanes(g, fn, l));
     if (!want || N > INT32_MAX) {
-        VG_CUDA(vg::launch_locate(g->d_desc, g->d_set, 1, N, prep, nullptr, g->sms, s));
+        VG_CUDA(vg::launch_locate(a, prep, g->sms, s));
         return VGRID_OK;
     }
     int rc = ensure_order(g, N);
     if (rc) return rc;
     const vg::RayOrder ord{g->d_bin, g->d_hist, g->d_order};
     VG_CUDA(cudaMemsetAsync(g->d_hist, 0, 2 * vg::kOrderBins * sizeof(uint32_t), s));
-    VG_CUDA(vg::launch_locate_ordered(g->d_desc, g->d_set, 1, N, ord, prep, g->sms, s));
+    a.bin = ord.bin;
+    a.hist = ord.hist;
+    VG_CUDA(vg::launch_locate(a, prep, g->sms, s));
     VG_CUDA(vg::launch_order(ord, N, g->sms, s));
     *order = g->d_order;
     return VGRID_OK;
@@ -861,15 +860,12 @@ int trace_tau_chunk(vgrid_t *g, const double *origin, const double *dir, int64_t
     const vgrid_launch L = shape_for(g, row, vg::MODE_TAU, n);
     const vg::KernelSet &ks = kernels(L.lanes_per_ray);
     RaySetDev set{origin, dir, tau, status, g->d_start, n, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, reset_stats ? g->d_stats : nullptr, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
-    if ((rc = locate_start(g, ks.get(row, vg::MODE_TAU), L, n, &order, s, fp64 != 0))) return rc;
+    if ((rc = locate_start(g, ks.get(row, vg::MODE_TAU), L, set, &order, s, fp64 != 0, reset_stats))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.grids = g->d_desc;
-    a.sets = g->d_set;
-    a.nsets = 1;
     a.total = n;
     a.queue = g->d_queue;
     a.stats = g->d_stats;
@@ -898,25 +894,25 @@ int trace_chunk_slot(vgrid_t *g, int k, const double *origin, const double *dir,
     VG_CUDA(cudaStreamWaitEvent(t, g->ev_in[k], 0));
     VG_CUDA(cudaStreamWaitEvent(t, g->ev_k[k], 0));
     RaySetDev set{origin, dir, tau, status, g->d_hstart[k], n, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_hset + k, set, g->d_hqueue + k, nullptr, t));
+    vg::LocateArgs la{g->d_desc, nullptr, 1, set, n, nullptr, nullptr, nullptr, g->d_hqueue + k, nullptr};
     const int prep = fp64 ? vg::PREP_FP64 : vg::PREP_FP32;
     const bool want = n <= INT32_MAX && (L.order == 1 || (L.order == 0 && n >= 2 * resident_lanes(g, fn, L)));
     const int32_t *order = nullptr;
     if (want) {
         const vg::RayOrder ord{g->d_hbin[k], g->d_hhist + 2 * vg::kOrderBins * k, g->d_horder[k]};
         VG_CUDA(cudaMemsetAsync(ord.hist, 0, 2 * vg::kOrderBins * sizeof(uint32_t), t));
-        VG_CUDA(vg::launch_locate_ordered(g->d_desc, g->d_hset + k, 1, n, ord, prep, g->sms, t));
+        la.bin = ord.bin;
+        la.hist = ord.hist;
+        VG_CUDA(vg::launch_locate(la, prep, g->sms, t));
         VG_CUDA(vg::launch_order(ord, n, g->sms, t));
         order = ord.order;
     } else {
-        VG_CUDA(vg::launch_locate(g->d_desc, g->d_hset + k, 1, n, prep, nullptr, g->sms, t));
+        VG_CUDA(vg::launch_locate(la, prep, g->sms, t));
     }
     VG_CUDA(cudaEventRecord(g->ev_prep[k], t));
     VG_CUDA(cudaStreamWaitEvent(s, g->ev_prep[k], 0));
     vg::TraceArgs a{};
     a.grids = g->d_desc;
-    a.sets = g->d_hset + k;
-    a.nsets = 1;
     a.total = n;
     a.queue = g->d_hqueue + k;
     a.stats = g->d_stats;
@@ -960,9 +956,8 @@ int vgrid_locate(vgrid_t *g, const double *pts, int64_t N, int precision, int32_
     cudaStream_t s = (cudaStream_t)stream;
     // the cells go straight to `cell`: no start records
     RaySetDev set{pts, pts, nullptr, nullptr, nullptr, N, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
-    VG_CUDA(vg::launch_locate(g->d_desc, g->d_set, 1, N,
-                              precision == VGRID_FP32_RECHECK ? vg::PREP_CELL32 : vg::PREP_CELL64, cell, g->sms, s));
+    const vg::LocateArgs la{g->d_desc, nullptr, 1, set, N, cell, nullptr, nullptr, nullptr, nullptr};
+    VG_CUDA(vg::launch_locate(la, precision == VGRID_FP32_RECHECK ? vg::PREP_CELL32 : vg::PREP_CELL64, g->sms, s));
     return VGRID_OK;
 }
 
@@ -1000,19 +995,16 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     const vgrid_launch L = shape_for(g, row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS, N, enter);
     const vg::KernelSet &ks = kernels(L.lanes_per_ray);
     RaySetDev set{origin, dir, tau, ray_status, g->d_start, N, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
     {
         const vg::TraceFn fn = ks.get(row, output == VGRID_TAU ? vg::MODE_TAU : vg::MODE_SEGS);
-        if ((rc = locate_start(g, fn, L, N, &order, s, fp64 != 0))) return rc;
+        if ((rc = locate_start(g, fn, L, set, &order, s, fp64 != 0))) return rc;
     }
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
     a.grids = g->d_desc;
-    a.sets = g->d_set;
-    a.nsets = 1;
     a.total = N;
     a.queue = g->d_queue;
     a.stats = g->d_stats;
@@ -1113,7 +1105,6 @@ int vgrid_trace_host(vgrid_t *g, const double *origin, const double *dir, int64_
     if (!g->s_h2d) {
         int rc = dmalloc(&g->d_hhist, 2 * 2 * vg::kOrderBins, g->device_bytes);
         if (!rc) rc = dmalloc(&g->d_hqueue, 2, g->device_bytes);
-        if (!rc) rc = dmalloc(&g->d_hset, 2, g->device_bytes);
         if (rc) return rc;
         VG_CUDA(cudaStreamCreateWithFlags(&g->s_h2d, cudaStreamNonBlocking));
         VG_CUDA(cudaStreamCreateWithFlags(&g->s_d2h, cudaStreamNonBlocking));
@@ -1212,18 +1203,15 @@ int vgrid_trace_grad(vgrid_t *g, const double *origin, const double *dir, int64_
     int rc = ensure_start(g, N);
     if (rc) return rc;
     RaySetDev set{origin, dir, nullptr, nullptr, g->d_start, N, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
     const vgrid_launch L = shape_for(g, 0, vg::MODE_GRAD, N);
     const vg::TraceFn fn = kernels(L.lanes_per_ray).get(0, vg::MODE_GRAD);
-    if ((rc = locate_start(g, fn, L, N, &order, s))) return rc;
+    if ((rc = locate_start(g, fn, L, set, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
     a.grids = g->d_desc;
-    a.sets = g->d_set;
-    a.nsets = 1;
     a.total = N;
     a.queue = g->d_queue;
     a.stats = g->d_stats;
@@ -1281,18 +1269,15 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
     int rc = ensure_start(g, N);
     if (rc) return rc;
     RaySetDev set{origin, dir, nullptr, nullptr, g->d_start, N, 0, 0, 0};
-    VG_CUDA(vg::launch_prepare(g->d_set, set, g->d_queue, g->d_stats, s));
     mark(g, 0, 0, s);
     const int32_t *order = nullptr;
     const vgrid_launch L = shape_for(g, 0, vg::MODE_INTERACT, N);
     const vg::TraceFn fn = kernels(L.lanes_per_ray).get(0, vg::MODE_INTERACT);
-    if ((rc = locate_start(g, fn, L, N, &order, s))) return rc;
+    if ((rc = locate_start(g, fn, L, set, &order, s))) return rc;
     mark(g, 0, 1, s);
     vg::TraceArgs a{};
     a.order = order;
     a.grids = g->d_desc;
-    a.sets = g->d_set;
-    a.nsets = 1;
     a.total = N;
     a.queue = g->d_queue;
     a.stats = g->d_stats;
@@ -1397,17 +1382,18 @@ int vgrid_batch_create(const vgrid_rayset *sets, int32_t G, const vgrid_launch *
 }
 
 static int batch_issue(vgrid_batch_t *b, cudaStream_t s) {
-    RaySetDev none{};
-    VG_CUDA(vg::launch_prepare(nullptr, none, b->d_queue, b->d_stats, s));
     vg::TraceArgs a{};
+    vg::LocateArgs la{b->d_grids, b->d_sets, b->G, {}, b->total, nullptr, nullptr, nullptr, b->d_queue, b->d_stats};
     if (b->launch.order == 1 && b->d_order) {
         const vg::RayOrder ord{b->d_bin, b->d_hist, b->d_order};
         VG_CUDA(cudaMemsetAsync(b->d_hist, 0, 2 * vg::kOrderBins * sizeof(uint32_t), s));
-        VG_CUDA(vg::launch_locate_ordered(b->d_grids, b->d_sets, b->G, b->total, ord, vg::PREP_FP32, b->sms, s));
+        la.bin = ord.bin;
+        la.hist = ord.hist;
+        VG_CUDA(vg::launch_locate(la, vg::PREP_FP32, b->sms, s));
         VG_CUDA(vg::launch_order(ord, b->total, b->sms, s));
         a.order = b->d_order;
     } else {
-        VG_CUDA(vg::launch_locate(b->d_grids, b->d_sets, b->G, b->total, vg::PREP_FP32, nullptr, b->sms, s));
+        VG_CUDA(vg::launch_locate(la, vg::PREP_FP32, b->sms, s));
     }
     a.grids = b->d_grids;
     a.sets = b->d_sets;

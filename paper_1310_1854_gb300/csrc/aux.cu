@@ -13,28 +13,10 @@ static std::atomic<int64_t> g_launches{0};
 void count_launches(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 int64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 
-// Write the ray-set descriptor and clear the work counter and statistics
-// (one thread; the descriptor travels as a kernel argument, so the call is
-// stream-ordered and needs no host staging buffer). stats may be NULL.
-__global__ void prepare_kernel(RaySetDev *d_set, RaySetDev set, unsigned long long *queue, StatsDev *stats) {
-    if (d_set) *d_set = set;
-    *queue = 0ull;
-    if (!stats) return;  // counters keep adding up (host-pipelined chunks)
-    unsigned long long *s = reinterpret_cast<unsigned long long *>(stats);
-    for (int i = 0; i < (int)(sizeof(StatsDev) / sizeof(unsigned long long)); i++) s[i] = 0ull;
-}
-
 __global__ void put_grid_kernel(GridDev *d, GridDev g) { *d = g; }
 
 cudaError_t launch_put_grid(GridDev *d, const GridDev &g, cudaStream_t s) {
     put_grid_kernel<<<1, 1, 0, s>>>(d, g);
-    count_launches(1);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_prepare(RaySetDev *d_set, const RaySetDev &set, unsigned long long *queue, StatsDev *stats,
-                           cudaStream_t s) {
-    prepare_kernel<<<1, 1, 0, s>>>(d_set, set, queue, stats);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -54,19 +36,27 @@ cudaError_t launch_prepare(RaySetDev *d_set, const RaySetDev &set, unsigned long
 // (10^7 points of the 10^6-site disk 426 -> 405 us; seven spill, 430).
 template <int PREP>
 __global__ void __launch_bounds__(256, PREP == PREP_CELL32 || PREP == PREP_CELL64 ? 6 : 5)
-    locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int32_t *out_caller,
-                  uint8_t *bin, uint32_t *hist) {
+    locate_kernel(const __grid_constant__ LocateArgs a) {
+    uint8_t *const bin = a.bin;
+    int32_t *const out_caller = a.out_caller;
+    // the work counter and the counters of the traversal that follows (a kernel
+    // of its own did this and stored the ray set before: about 3 us per call)
+    if (blockIdx.x == 0) {
+        constexpr int kCounters = sizeof(StatsDev) / sizeof(unsigned long long);
+        if (a.stats && threadIdx.x < kCounters) reinterpret_cast<unsigned long long *>(a.stats)[threadIdx.x] = 0ull;
+        if (a.queue && threadIdx.x == kCounters) *a.queue = 0ull;
+    }
     __shared__ uint32_t s_hist[kOrderBins];
     if (bin) {
         for (int b = threadIdx.x; b < kOrderBins; b += blockDim.x) s_hist[b] = 0u;
         __syncthreads();
     }
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
-        const int set = find_set(sets, nsets, w);
-        const RaySetDev &rs = sets[set];
-        const int64_t li = w - rs.first;
-        const GridDev *gp = grids + rs.grid;
-        const double *o = rs.origin + 3 * li;
+    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < a.total;
+         w += (int64_t)gridDim.x * blockDim.x) {
+        const RaySetDev *rs = a.sets ? a.sets + find_set(a.sets, a.nsets, w) : &a.one;
+        const int64_t li = w - rs->first;
+        const GridDev *gp = a.grids + rs->grid;
+        const double *o = rs->origin + 3 * li;
         const LocPt P = loc_point(__ldg(o), __ldg(o + 1), __ldg(o + 2));
         // float32 distances with the proven float64 fallback give exactly the
         // float64 argmin, so both traversal forms start that way; only
@@ -74,8 +64,8 @@ __global__ void __launch_bounds__(256, PREP == PREP_CELL32 || PREP == PREP_CELL6
         int m = locate_point<true>(gp, P, PREP != PREP_CELL64, nullptr);
         if (out_caller) out_caller[w] = m >= 0 ? __ldg(&gp->perm[m]) : -1;
         if (PREP == PREP_CELL32 || PREP == PREP_CELL64) continue;
-        RayPrep *out = rs.start + li;
-        const double *d = rs.dir + 3 * li;
+        RayPrep *out = rs->start + li;
+        const double *d = rs->dir + 3 * li;
         const double k[3] = {__ldg(d), __ldg(d + 1), __ldg(d + 2)};
         RayPrep p;
         for (int c = 0; c < 3; c++) {
@@ -205,31 +195,28 @@ __global__ void __launch_bounds__(256, PREP == PREP_CELL32 || PREP == PREP_CELL6
     if (bin) {
         __syncthreads();
         for (int b = threadIdx.x; b < kOrderBins; b += blockDim.x)
-            if (s_hist[b]) atomicAdd(&hist[b], s_hist[b]);
+            if (s_hist[b]) atomicAdd(&a.hist[b], s_hist[b]);
     }
 }
 
-static cudaError_t launch_locate_kernel(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
-                                        int32_t *out_caller, uint8_t *bin, uint32_t *hist, int sms, cudaStream_t s) {
-    if (total <= 0) return cudaSuccess;
+cudaError_t launch_locate(const LocateArgs &a, int prep, int sms, cudaStream_t s) {
+    if (a.total <= 0) {
+        cudaError_t e = a.queue ? cudaMemsetAsync(a.queue, 0, sizeof(*a.queue), s) : cudaSuccess;
+        if (e == cudaSuccess && a.stats) e = cudaMemsetAsync(a.stats, 0, sizeof(*a.stats), s);
+        return e;
+    }
     // many more blocks than fit: points differ in the records they scan, and the
     // blocks that end early make room (8 / 16 / 32 / 64 per SM and one point per
     // thread took 457 / 452 / 422 / 418 / 435 us for the same points)
-    const int64_t blocks = std::min<int64_t>((total + 255) / 256, (int64_t)sms * 64);
-    const dim3 g((unsigned)blocks);
+    const dim3 g((unsigned)std::min<int64_t>((a.total + 255) / 256, (int64_t)sms * 64));
     switch (prep) {
-        case PREP_CELL32: locate_kernel<PREP_CELL32><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
-        case PREP_CELL64: locate_kernel<PREP_CELL64><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
-        case PREP_FP64: locate_kernel<PREP_FP64><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
-        default: locate_kernel<PREP_FP32><<<g, 256, 0, s>>>(grids, sets, nsets, total, out_caller, bin, hist); break;
+        case PREP_CELL32: locate_kernel<PREP_CELL32><<<g, 256, 0, s>>>(a); break;
+        case PREP_CELL64: locate_kernel<PREP_CELL64><<<g, 256, 0, s>>>(a); break;
+        case PREP_FP64: locate_kernel<PREP_FP64><<<g, 256, 0, s>>>(a); break;
+        default: locate_kernel<PREP_FP32><<<g, 256, 0, s>>>(a); break;
     }
     count_launches(1);
     return cudaGetLastError();
-}
-
-cudaError_t launch_locate_ordered(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total,
-                                  const RayOrder &ord, int prep, int sms, cudaStream_t s) {
-    return launch_locate_kernel(grids, sets, nsets, total, prep, nullptr, ord.bin, ord.hist, sms, s);
 }
 
 // cursor[b] = number of rays in longer bins (the longest bin goes first)
@@ -287,11 +274,6 @@ cudaError_t launch_order(const RayOrder &ord, int64_t total, int sms, cudaStream
                                                                      ord.order);
     count_launches(1);
     return cudaGetLastError();
-}
-
-cudaError_t launch_locate(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
-                          int32_t *out_caller, int sms, cudaStream_t s) {
-    return launch_locate_kernel(grids, sets, nsets, total, prep, out_caller, nullptr, nullptr, sms, s);
 }
 
 // rho (caller order) into the headers of both forms of the cell blocks

@@ -99,8 +99,6 @@ int64_t launches_so_far();
 cudaError_t launch_put_grid(GridDev *d, const GridDev &g, cudaStream_t s);
 cudaError_t launch_enter(const double *origin, const double *dir, int64_t N, const GridDev *gp, double *out, int sms,
                          cudaStream_t s);
-cudaError_t launch_prepare(RaySetDev *d_set, const RaySetDev &set, unsigned long long *queue, StatsDev *stats,
-                           cudaStream_t s);
 // what the start-cell kernel writes per ray (see locate_kernel)
 enum { PREP_CELL32 = 0, PREP_FP32 = 1, PREP_FP64 = 2, PREP_CELL64 = 3 };
 // Longest-predicted-first ray order. A persistent launch ends when its last
@@ -120,13 +118,26 @@ struct RayOrder {
     uint32_t *hist;   // kOrderBins counts, then kOrderBins cursors (zeroed by the caller)
     int32_t *order;   // queue position -> ray
 };
-// the start records (PREP_FP32 or PREP_FP64) plus the bins and their counts
-cudaError_t launch_locate_ordered(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total,
-                                  const RayOrder &ord, int prep, int sms, cudaStream_t s);
+// One launch of the start-cell kernel. sets: device, nsets of them, or NULL for
+// the one set `one`. bin, hist: with them the ray order's bins and their counts
+// come too (PREP_FP32 and PREP_FP64). queue, stats: cleared for the traversal
+// that follows on the stream (nullable: host-pipelined chunks keep adding up
+// their counters).
+struct LocateArgs {
+    const GridDev *grids;
+    const RaySetDev *sets;
+    int32_t nsets;
+    RaySetDev one;
+    int64_t total;
+    int32_t *out_caller;
+    uint8_t *bin;
+    uint32_t *hist;
+    unsigned long long *queue;
+    StatsDev *stats;
+};
+cudaError_t launch_locate(const LocateArgs &a, int prep, int sms, cudaStream_t s);
 // bins -> permutation (scan of the counts, longest bin first, and scatter)
 cudaError_t launch_order(const RayOrder &ord, int64_t total, int sms, cudaStream_t s);
-cudaError_t launch_locate(const GridDev *grids, const RaySetDev *sets, int nsets, int64_t total, int prep,
-                          int32_t *out_caller, int sms, cudaStream_t s);
 cudaError_t launch_permute_density(const float *rho_caller, const int32_t *perm, const float4 *site, int64_t M,
                                    float4 *cells, float4 *rel, cudaStream_t s);
 // Device arrays of a grid from its cells (layout.cu), on the current device.

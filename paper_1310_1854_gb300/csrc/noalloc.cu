@@ -4,7 +4,7 @@
 // allocator with a fixed budget, or they run latency-bound loops that must
 // not take the implicit device synchronisation of cudaMalloc/cudaFree. For
 // them the work buffers of the traversal (start cells, work counter,
-// counters, ray-set descriptor) live in one file-scope device array of fixed
+// counters) live in one file-scope device array of fixed
 // size instead of buffers allocated per grid. The array exists once per
 // device that loads the library and stays until the process exits.
 #include <cuda_runtime.h>
@@ -21,10 +21,8 @@ namespace {
 // layout of the scratch array
 constexpr size_t kQueueOff = 0;     // unsigned long long work counter
 constexpr size_t kStatsOff = 64;    // StatsDev
-constexpr size_t kSetOff = 256;     // RaySetDev
 constexpr size_t kStartOff = 512;   // RayPrep start record per ray
-static_assert(sizeof(StatsDev) <= kSetOff - kStatsOff, "stats slot");
-static_assert(sizeof(RaySetDev) <= kStartOff - kSetOff, "ray-set slot");
+static_assert(sizeof(StatsDev) <= kStartOff - kStatsOff, "stats slot");
 static_assert(sizeof(RayPrep) == 64, "start record");
 static_assert(kStartOff + sizeof(RayPrep) * (size_t)VGRID_NOALLOC_MAX_RAYS == (size_t)VGRID_NOALLOC_SCRATCH_BYTES, "size");
 
@@ -81,15 +79,13 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
         }
         auto *queue = reinterpret_cast<unsigned long long *>(base + kQueueOff);
         auto *stats = reinterpret_cast<StatsDev *>(base + kStatsOff);
-        auto *dset = reinterpret_cast<RaySetDev *>(base + kSetOff);
         auto *start = reinterpret_cast<RayPrep *>(base + kStartOff);
         cudaStream_t s = (cudaStream_t)stream;
         const int fp64 = precision == VGRID_FP64;
         RaySetDev set{origin, dir, tau, ray_status, start, N, 0, 0, 0};
         // clears the counter and statistics left by the previous call
-        if ((e = vg::launch_prepare(dset, set, queue, stats, s)) != cudaSuccess ||
-            (e = vg::launch_locate(v.d_desc, dset, 1, N, fp64 ? vg::PREP_FP64 : vg::PREP_FP32, nullptr, v.sms,
-                                   s)) != cudaSuccess) {
+        const vg::LocateArgs la{v.d_desc, nullptr, 1, set, N, nullptr, nullptr, nullptr, queue, stats};
+        if ((e = vg::launch_locate(la, fp64 ? vg::PREP_FP64 : vg::PREP_FP32, v.sms, s)) != cudaSuccess) {
             rc = fail(VGRID_ERR_CUDA, cudaGetErrorString(e));
             break;
         }
@@ -97,8 +93,6 @@ extern "C" int vgrid_trace_noalloc(vgrid_t *g, const double *origin, const doubl
         const vg::TraceFn fn = vg::pick_trace(g, precision == VGRID_FP32_EXACT ? 2 : fp64, N, &block, &blocks);
         vg::TraceArgs a{};
         a.grids = v.d_desc;
-        a.sets = dset;
-        a.nsets = 1;
         a.total = N;
         a.queue = queue;
         a.stats = stats;
