@@ -785,7 +785,10 @@ int precision_row(int precision) {
 // / 1229. Rays that enter from outside cross the whole domain and are more alike
 // still, so that throughput counts from fewer of them on: 10^4 into a ball of
 // 60,000 sites 228 / 188 / 153 / 138, 30,000 278 / 220 / 209 / 253, 50,000 294 / 262 /
-// 307 / 343, 75,000 315 / 330 / 364 / 476. The float64 form repeats its float64 work in every lane, so it takes
+// 307 / 343, 75,000 315 / 330 / 364 / 476. Parallel rays of a detector, started
+// on the domain's face, are like them but cannot be told from others here: eight
+// lanes stop at 0.22 R, where they lose little (30,600 of them through a ball,
+// forward and adjoint, 959 / 928 / 985 / 1233). The float64 form repeats its float64 work in every lane, so it takes
 // more than one only for very few rays (10^4 rays on 1000 sites: 128 / 111 / 133 /
 // 172) and where one lane each would leave a short second wave (10^5 on the disk:
 // 1630 / 1324), and single-warp blocks while they do not fill the SMs (the
@@ -803,7 +806,7 @@ vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N, bool ente
         L.lanes_per_ray = N <= 0.04 * R ? 8 : N <= 0.15 * R || (N > R && N <= 1.25 * R) ? 2 : 1;
         if (N * L.lanes_per_ray < R) L.block = 32;
     } else {
-        const double f8 = enter ? 0.11 : 0.4, f4 = enter ? 0.27 : 0.75, f2 = enter ? 0.45 : 1.4;
+        const double f8 = enter ? 0.11 : 0.22, f4 = enter ? 0.27 : 0.75, f2 = enter ? 0.45 : 1.4;
         L.lanes_per_ray = N <= f8 * R ? 8 : N <= f4 * R ? 4 : N <= f2 * R ? 2 : 1;
     }
     return L;
