@@ -67,8 +67,9 @@ class VoronoiGrid:
     """A Voronoi grid on the current CUDA device.
 
     sites: (M, 3) array of float32-representable positions inside ``box``
-    (xmin, ymin, zmin, xmax, ymax, zmax). The neighbour lists, cell volumes,
-    bounding boxes and block lists are built on the host by the library.
+    (xmin, ymin, zmin, xmax, ymax, zmax). The neighbour lists, cell volumes
+    and bounding boxes are built by the library, on the host or with ``gpu_build``
+    on the GPU, the block lists and the traversal's cell blocks on the GPU.
     ``sphere=(cx, cy, cz, R)`` makes the domain that ball (inside ``box``,
     every site inside it): paths end on the sphere, points outside it are
     outside the domain.
