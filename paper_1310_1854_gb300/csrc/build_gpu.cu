@@ -82,17 +82,40 @@ __device__ __forceinline__ int bucket_coord(double v, const double *edge, int di
 
 // The grid lines of one axis: edge[i] is the (i n / dim)-th smallest of the n
 // sampled coordinates (every stride-th site's; float32 values), the box bounds
-// at both ends. One block per line: the value whose rank it is, found bit by
-// bit, each step counting the sample. Sorting the three samples on the host
-// took 10 of the 37 ms of the cell phase at 10^5 sites.
+// at both ends. One block per line finds the value whose rank it is, two bits at
+// a time, each step counting the sample below three thresholds. Sorting the three
+// samples on the host took 10 of the 37 ms of the cell phase at 10^5 sites.
+// The counting is bound by the reads of the sample from L2, so it is laid out
+// as one array of keys per axis (4 bytes a site instead of a strided float4),
+// read 16 bytes a thread by 1024 threads; with one bit per step over the sites
+// themselves and 256 threads it took 1006 us at 10^5 sites, 80 now.
+constexpr int kLineThreads = 1024;
+
 __device__ __forceinline__ unsigned float_order(float x) {  // orders like the value
     const unsigned b = __float_as_uint(x);
     return (b & 0x80000000u) ? ~b : b | 0x80000000u;
 }
 
-__global__ void __launch_bounds__(256) grid_lines_kernel(const float4 *Sf, int64_t stride, int n, int3 dims, double3 lo,
-                                                         double3 hi, double *edge) {
-    __shared__ int s_count[8];
+// keys[c n4 + k]: coordinate c of sample k; n4 is n rounded up to a multiple of
+// four, the rest of each array the largest key, which is below no threshold
+__global__ void sample_keys_kernel(const float4 *Sf, int64_t stride, int n, int n4, unsigned *keys) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n4) return;
+    unsigned x = 0xffffffffu, y = x, z = x;
+    if (k < n) {
+        const float4 q = __ldg(Sf + k * stride);
+        x = float_order(q.x);
+        y = float_order(q.y);
+        z = float_order(q.z);
+    }
+    keys[k] = x;
+    keys[n4 + k] = y;
+    keys[2 * n4 + k] = z;
+}
+
+__global__ void __launch_bounds__(kLineThreads) grid_lines_kernel(const unsigned *keys, int n, int n4, int3 dims,
+                                                                  double3 lo, double3 hi, double *edge) {
+    __shared__ int s_count[3][kLineThreads / 32];
     const int dim[3] = {dims.x, dims.y, dims.z};
     int i = blockIdx.x, c = 0, first = 0;  // line i of axis c, dim + 1 lines each
     while (i > dim[c]) {
@@ -106,22 +129,36 @@ __global__ void __launch_bounds__(256) grid_lines_kernel(const float4 *Sf, int64
         return;
     }
     const int rank = (int)((int64_t)i * n / dim[c]);
+    const uint4 *q4 = reinterpret_cast<const uint4 *>(keys + (int64_t)c * n4);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the largest key with at most `rank` keys below it
     unsigned key = 0u;
-    for (int bit = 31; bit >= 0; bit--) {
-        const unsigned t = key | (1u << bit);
-        int below = 0;
-        for (int k = threadIdx.x; k < n; k += 256) {
-            const float4 q = __ldg(Sf + k * stride);
-            below += float_order(c == 0 ? q.x : c == 1 ? q.y : q.z) < t;
+    for (int bit = 30; bit >= 0; bit -= 2) {
+        const unsigned t1 = key | (1u << bit), t2 = key | (2u << bit), t3 = key | (3u << bit);
+        int b1 = 0, b2 = 0, b3 = 0;
+#pragma unroll 4
+        for (int k = threadIdx.x; k < n4 / 4; k += kLineThreads) {
+            const uint4 q = __ldg(q4 + k);
+            b1 += (q.x < t1) + (q.y < t1) + (q.z < t1) + (q.w < t1);
+            b2 += (q.x < t2) + (q.y < t2) + (q.z < t2) + (q.w < t2);
+            b3 += (q.x < t3) + (q.y < t3) + (q.z < t3) + (q.w < t3);
         }
-        below = __reduce_add_sync(0xffffffffu, below);
-        if ((threadIdx.x & 31) == 0) s_count[threadIdx.x >> 5] = below;
+        b1 = __reduce_add_sync(0xffffffffu, b1);
+        b2 = __reduce_add_sync(0xffffffffu, b2);
+        b3 = __reduce_add_sync(0xffffffffu, b3);
+        if (lane == 0) {
+            s_count[0][warp] = b1;
+            s_count[1][warp] = b2;
+            s_count[2][warp] = b3;
+        }
         __syncthreads();
-        int all = 0;
-        for (int w = 0; w < 8; w++) all += s_count[w];
+        // every warp adds the warps' counts up for itself
+        static_assert(kLineThreads == 1024, "one lane per warp's count");
+        b1 = __reduce_add_sync(0xffffffffu, s_count[0][lane]);
+        b2 = __reduce_add_sync(0xffffffffu, s_count[1][lane]);
+        b3 = __reduce_add_sync(0xffffffffu, s_count[2][lane]);
         __syncthreads();
-        if (all <= rank) key = t;
+        key = b3 <= rank ? t3 : b2 <= rank ? t2 : b1 <= rank ? t1 : key;
     }
     if (threadIdx.x == 0) {
         const float v = __uint_as_float((key & 0x80000000u) ? key & 0x7fffffffu : ~key);
@@ -667,10 +704,16 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         if ((e = cudaMemcpy(dSf, sf.data(), sizeof(float4) * M, cudaMemcpyHostToDevice)) != cudaSuccess)
             return bad(e, "upload");
     }
-    grid_lines_kernel<<<(unsigned)lines, 256>>>(dSf, stride, (int)((M + stride - 1) / stride),
-                                                make_int3(bg.dim[0], bg.dim[1], bg.dim[2]),
-                                                make_double3(box[0], box[1], box[2]),
-                                                make_double3(box[3], box[4], box[5]), dE);
+    {
+        // the keys lie in the lists' buffer (64 M ints), which the cells fill later
+        static_assert(kCap >= 12, "3 (n + 3) keys, n <= M");
+        const int n = (int)((M + stride - 1) / stride), n4 = (n + 3) & ~3;
+        unsigned *const keys = reinterpret_cast<unsigned *>(nbr);
+        sample_keys_kernel<<<(unsigned)((n4 + 255) / 256), 256>>>(dSf, stride, n, n4, keys);
+        grid_lines_kernel<<<(unsigned)lines, kLineThreads>>>(keys, n, n4, make_int3(bg.dim[0], bg.dim[1], bg.dim[2]),
+                                                             make_double3(box[0], box[1], box[2]),
+                                                             make_double3(box[3], box[4], box[5]), dE);
+    }
     if ((e = cudaMemset(boff, 0, sizeof(int64_t) * (K + 1))) != cudaSuccess) return bad(e, "memset");
     const int blocks = (int)std::min<int64_t>((M + 255) / 256, 65535);
     bucket_count_kernel<<<blocks, 256>>>(dS, M, bg, bidx, boff);
@@ -693,7 +736,7 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
     if ((e = cudaMemset(cursor, 0, sizeof(unsigned long long))) != cudaSuccess) return bad(e, "memset");
     cells_kernel<<<cblocks, 128>>>(dS, M, bg, boff, bsites, box[0], box[1], box[2], box[3], box[4], box[5], eps, cnt,
                                    nbr, vol, bbox, fail, reinterpret_cast<unsigned long long *>(cursor), dSf, lanes);
-    count_launches(5);  // grid lines, bucket count, fill, sort, cells (the scan counts its own)
+    count_launches(6);  // keys, grid lines, bucket count, fill, sort, cells (the scan counts its own)
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bad(e, "cells kernel");
     std::vector<int> hcnt(M), hfail(M);
     out.vol.assign(M, 0.0);
