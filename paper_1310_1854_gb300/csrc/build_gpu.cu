@@ -13,9 +13,8 @@
 // gives every bucket about the same number of sites. One thread builds one cell: a convex polyhedron in
 // float64 with shared vertices and faces as vertex loops, cut plane by plane
 // while the buckets are visited ring by ring around the site, the sites of
-// each ring nearest first. Fixed capacities keep the polyhedron in local
-// memory; a cell that would overflow them is flagged and rebuilt by the
-// host builder.
+// each ring nearest first. The polyhedron has fixed capacities; a cell that
+// would overflow them is flagged and rebuilt by the host builder.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,32 +40,41 @@ struct BucketGrid {
     int dim[3];
 };
 
-struct DPoly {
-    double x[kNV], y[kNV], z[kNV];
-    int nv;
-    int fid[kNF];
-    short fbeg[kNF], flen[kNF];
-    int nf;
-    unsigned char L[kNL];
-    int nl;
+struct Face {
+    int id;
+    short beg, len;
 };
 
-struct Scratch {
-    double fv[kNV];
-    int fid[kNF];
-    short fbeg[kNF], flen[kNF];
+constexpr int kBuf = 384;  // candidates of one drain
+
+// A thread's polyhedron and scratch: a run of global memory of its own. Local
+// memory deals the threads' 4-byte words out in turn, so with the lanes of a warp
+// at different cells (about 4 of 32 run together) every access moved a 32-byte
+// sector for 4 bytes of it: 80 GB of DRAM traffic for 2 10^5 clumpy cells, 24 now,
+// L1 hits 46 -> 81 %. Cell kernel 23.6 -> 15.8 ms at 10^5 clumpy sites, cell phase
+// 138 -> 107 ms at 10^6. (32-byte vertices moved as pairs of double2: 2 % slower.)
+struct Cell {
+    struct {
+        double x, y, z, f;  // f: the value of the cutting plane
+    } v[kNV];
+    Face face[kNF];
     unsigned char L[kNL];
-    unsigned char seg_a[kNF], seg_b[kNF];
+    unsigned long long key[kBuf];  // candidates: distance bits above the site
+    // scratch of a cut
+    union {
+        struct {
+            double x, y, z;
+        } w[kNV];              // the vertices kept by a cut
+        float far[3 * kNV];    // between cuts: the vertices a candidate can still cut
+    };
+    Face face2[kNF];
+    unsigned char L2[kNL];
     int ekey[kNE];
     unsigned char evid[kNE];
     unsigned char remap[kNV];
-    union {
-        struct {
-            double x[kNV], y[kNV], z[kNV];  // the vertices kept by a cut
-        };
-        float far[3 * kNV];                 // between cuts: the vertices a candidate can still cut
-    };
+    unsigned char seg_a[kNF], seg_b[kNF];
 };
+static_assert(sizeof(Cell) % 32 == 0, "every cell starts on a sector");
 
 // the bucket of coordinate v along one axis: the largest i < dim with
 // edge[i] <= v (0 below the first line)
@@ -200,21 +208,24 @@ __global__ void bucket_sort_kernel(const int64_t *off, int64_t K, int *bsites) {
     }
 }
 
-__device__ void poly_box(DPoly &P, const double *box) {
-    P.nv = 8;
+// counts of the polyhedron, in registers
+struct Counts {
+    int nv, nf, nl;
+};
+
+__device__ void poly_box(Cell &P, Counts &C, const double *box) {
+    C.nv = 8;
     for (int i = 0; i < 8; i++) {
-        P.x[i] = (i & 4) ? box[3] : box[0];
-        P.y[i] = (i & 2) ? box[4] : box[1];
-        P.z[i] = (i & 1) ? box[5] : box[2];
+        P.v[i].x = (i & 4) ? box[3] : box[0];
+        P.v[i].y = (i & 2) ? box[4] : box[1];
+        P.v[i].z = (i & 1) ? box[5] : box[2];
     }
     // counter-clockwise seen from outside; walls -1..-6 = x min, x max, y min, y max, z min, z max
     const unsigned char quad[6][4] = {{0, 1, 3, 2}, {4, 6, 7, 5}, {0, 4, 5, 1}, {2, 3, 7, 6}, {0, 2, 6, 4}, {1, 5, 7, 3}};
-    P.nf = 6;
-    P.nl = 24;
+    C.nf = 6;
+    C.nl = 24;
     for (int w = 0; w < 6; w++) {
-        P.fid[w] = -(w + 1);
-        P.fbeg[w] = (short)(4 * w);
-        P.flen[w] = 4;
+        P.face[w] = Face{-(w + 1), (short)(4 * w), 4};
         for (int k = 0; k < 4; k++) P.L[4 * w + k] = quad[w][k];
     }
 }
@@ -230,7 +241,7 @@ __device__ __forceinline__ float trunc_float(double x) {
 
 // Cut P by {x : n.x <= d}. 1: changed, 0: untouched, -1: capacity exceeded
 // or topology broken (the caller rebuilds the cell on the host).
-__device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, double d, int id, double eps) {
+__device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, double d, int id, double eps) {
     // each vertex classified once: above the plane (fv > eps) and strictly
     // below it (fv < -eps) as bits of two 128-bit masks held in registers,
     // so that the face walk below tests the masks and reads fv only at the
@@ -239,9 +250,9 @@ __device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, d
     static_assert(kNV <= 128, "vertex masks hold 128 bits");
     unsigned long long out0 = 0ull, out1 = 0ull, str0 = 0ull, str1 = 0ull;
     const long long eb = __double_as_longlong(eps);
-    for (int i = 0; i < P.nv; i++) {
-        const double f = nx * P.x[i] + ny * P.y[i] + nz * P.z[i] - d;
-        W.fv[i] = f;
+    for (int i = 0; i < C.nv; i++) {
+        const double f = nx * P.v[i].x + ny * P.v[i].y + nz * P.v[i].z - d;
+        P.v[i].f = f;
         const long long fb = __double_as_longlong(f);
         const unsigned long long bit = 1ull << (i & 63);
         const unsigned long long ob = fb > eb ? bit : 0ull;
@@ -257,21 +268,23 @@ __device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, d
     if (!(out0 | out1)) return 0;
     auto is_out = [&](int v) { return ((v < 64 ? out0 >> v : out1 >> (v - 64)) & 1ull) != 0ull; };
     auto is_strict = [&](int v) { return ((v < 64 ? str0 >> v : str1 >> (v - 64)) & 1ull) != 0ull; };
-    int ne = 0, nseg = 0, nf2 = 0, nl2 = 0, nv = P.nv;
-    for (int f = 0; f < P.nf; f++) {
-        const int b = P.fbeg[f], k = P.flen[f];
-        int out_count = 0;
-        for (int i = 0; i < k; i++) out_count += is_out(P.L[b + i]);
-        if (out_count == k) continue;
-        if (nf2 >= kNF) return -1;
+    int ne = 0, nseg = 0, nf2 = 0, nl2 = 0, nv = C.nv;
+    for (int f = 0; f < C.nf; f++) {
+        const Face fc = P.face[f];
+        const int b = fc.beg, k = fc.len;
         const int start = nl2;
         int entry = -1, exit_ = -1;
-        for (int i = 0; i < k; i++) {
-            const int va = P.L[b + i], vb = P.L[b + (i + 1) % k];
-            const bool ao = is_out(va), bo = is_out(vb);
+        // one pass: a face wholly above the plane leaves no entries
+        int vb = P.L[b];
+        bool bo = is_out(vb);
+        for (int i = 1; i <= k; i++) {
+            const int va = vb;
+            const bool ao = bo;
+            vb = P.L[b + (i < k ? i : 0)];
+            bo = is_out(vb);
             if (!ao) {
                 if (nl2 >= kNL) return -1;
-                W.L[nl2++] = (unsigned char)va;
+                P.L2[nl2++] = (unsigned char)va;
             }
             if (ao != bo) {
                 const bool strict = !ao ? is_strict(va) : is_strict(vb);
@@ -282,21 +295,21 @@ __device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, d
                     const int key = lo * 256 + hi;
                     x = -1;
                     for (int e = 0; e < ne; e++)
-                        if (W.ekey[e] == key) { x = W.evid[e]; break; }
+                        if (P.ekey[e] == key) { x = P.evid[e]; break; }
                     if (x < 0) {
                         if (ne >= kNE || nv >= kNV) return -1;
-                        const double t = W.fv[lo] / (W.fv[lo] - W.fv[hi]);
-                        P.x[nv] = P.x[lo] + t * (P.x[hi] - P.x[lo]);
-                        P.y[nv] = P.y[lo] + t * (P.y[hi] - P.y[lo]);
-                        P.z[nv] = P.z[lo] + t * (P.z[hi] - P.z[lo]);
-                        W.fv[nv] = 0.0;
-                        W.ekey[ne] = key;
-                        W.evid[ne] = (unsigned char)nv;
+                        const auto vl = P.v[lo], vh = P.v[hi];
+                        const double t = vl.f / (vl.f - vh.f);
+                        P.v[nv].x = vl.x + t * (vh.x - vl.x);
+                        P.v[nv].y = vl.y + t * (vh.y - vl.y);
+                        P.v[nv].z = vl.z + t * (vh.z - vl.z);
+                        P.ekey[ne] = key;
+                        P.evid[ne] = (unsigned char)nv;
                         ne++;
                         x = nv++;
                     }
                     if (nl2 >= kNL) return -1;
-                    W.L[nl2++] = (unsigned char)x;
+                    P.L2[nl2++] = (unsigned char)x;
                 }
                 if (!ao) exit_ = x;
                 else entry = x;
@@ -304,15 +317,13 @@ __device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, d
         }
         if (entry >= 0 && exit_ >= 0 && entry != exit_) {
             if (nseg >= kNF) return -1;
-            W.seg_a[nseg] = (unsigned char)entry;
-            W.seg_b[nseg] = (unsigned char)exit_;
+            P.seg_a[nseg] = (unsigned char)entry;
+            P.seg_b[nseg] = (unsigned char)exit_;
             nseg++;
         }
+        if (nl2 > start && nf2 >= kNF) return -1;
         if (nl2 - start >= 3) {
-            W.fid[nf2] = P.fid[f];
-            W.fbeg[nf2] = (short)start;
-            W.flen[nf2] = (short)(nl2 - start);
-            nf2++;
+            P.face2[nf2++] = Face{fc.id, (short)start, (short)(nl2 - start)};
         } else {
             nl2 = start;
         }
@@ -320,74 +331,70 @@ __device__ int poly_cut(DPoly &P, Scratch &W, double nx, double ny, double nz, d
     if (nseg > 0) {
         // cap face: chain the cut segments entry -> exit
         const int start = nl2;
-        int cur = W.seg_a[0];
+        int cur = P.seg_a[0];
         const int first = cur;
         bool ok = true;
         unsigned long long used = 0ull;
         for (int step = 0; step < nseg; step++) {
             int pick = -1;
             for (int i = 0; i < nseg; i++)
-                if (!((used >> i) & 1ull) && W.seg_a[i] == cur) { pick = i; break; }
+                if (!((used >> i) & 1ull) && P.seg_a[i] == cur) { pick = i; break; }
             if (pick < 0) { ok = false; break; }
             used |= 1ull << pick;
             if (nl2 >= kNL) return -1;
-            W.L[nl2++] = W.seg_a[pick];
-            cur = W.seg_b[pick];
+            P.L2[nl2++] = P.seg_a[pick];
+            cur = P.seg_b[pick];
         }
         if (!ok || cur != first) return -1;  // inconsistent topology: leave it to the host
         if (nl2 - start >= 3) {
             if (nf2 >= kNF) return -1;
-            W.fid[nf2] = id;
-            W.fbeg[nf2] = (short)start;
-            W.flen[nf2] = (short)(nl2 - start);
-            nf2++;
+            P.face2[nf2++] = Face{id, (short)start, (short)(nl2 - start)};
         } else {
             nl2 = start;
         }
     }
     // compact the vertices that are still referenced
-    for (int i = 0; i < nv; i++) W.remap[i] = 255;
+    for (int i = 0; i < nv; i++) P.remap[i] = 255;
     int nv2 = 0;
     for (int i = 0; i < nl2; i++) {
-        const int v = W.L[i];
-        if (W.remap[v] == 255) {
-            W.remap[v] = (unsigned char)nv2;
-            W.x[nv2] = P.x[v];
-            W.y[nv2] = P.y[v];
-            W.z[nv2] = P.z[v];
-            nv2++;
+        const int v = P.L2[i];
+        int r = P.remap[v];
+        if (r == 255) {
+            r = nv2++;
+            P.remap[v] = (unsigned char)r;
+            P.w[r].x = P.v[v].x;
+            P.w[r].y = P.v[v].y;
+            P.w[r].z = P.v[v].z;
         }
-        P.L[i] = W.remap[v];
+        P.L[i] = (unsigned char)r;
     }
     for (int i = 0; i < nv2; i++) {
-        P.x[i] = W.x[i];
-        P.y[i] = W.y[i];
-        P.z[i] = W.z[i];
+        P.v[i].x = P.w[i].x;
+        P.v[i].y = P.w[i].y;
+        P.v[i].z = P.w[i].z;
     }
-    P.nv = nv2;
-    P.nl = nl2;
-    P.nf = nf2;
-    for (int f = 0; f < nf2; f++) {
-        P.fid[f] = W.fid[f];
-        P.fbeg[f] = W.fbeg[f];
-        P.flen[f] = W.flen[f];
-    }
+    C.nv = nv2;
+    C.nl = nl2;
+    C.nf = nf2;
+    for (int f = 0; f < nf2; f++) P.face[f] = P.face2[f];
     return nf2 >= 4 ? 1 : -1;
 }
 
 // Persistent threads: each takes its next cell from a global counter as soon
 // as it has finished one, so a thread whose cell needed few cuts does not
 // wait for the slowest cell of its block. Eight blocks of 128 per SM (64
-// registers): the kernel waits on its local-memory polyhedra and gains more
-// from the extra warps than it loses to the few more spills.
+// registers): the kernel waits on its polyhedra and gains more from the extra
+// warps than it loses to the spills where cells are many (10^6 clumpy sites: 105 ms, 111 with six
+// blocks, 117 with five; 10^5: 20.9, 19.4 and 19.3).
 __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t M, BucketGrid bg, const int64_t *boff,
                                                     const int *bsites, double box0, double box1, double box2,
                                                     double box3, double box4, double box5, double eps, int *out_cnt,
                                                     int *out_nbr, double *out_vol, double *out_bbox, int *out_fail,
-                                                    unsigned long long *next, const float4 *Sf, int lanes) {
+                                                    unsigned long long *next, const float4 *Sf, int lanes,
+                                                    Cell *pool) {
     if ((int)(threadIdx.x & 31) >= lanes) return;  // few cells: fewer lanes in more warps (see the launch)
-    DPoly P;
-    Scratch W;
+    Cell &P = pool[(int64_t)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * lanes + (threadIdx.x & 31)];
+    Counts C;
     const double box[6] = {box0, box1, box2, box3, box4, box5};
     double X = 0.0;
     for (int c = 0; c < 6; c++) X = fmax(X, fabs(box[c]));
@@ -395,7 +402,7 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
     const float off = Xf * 0x1p-19f;  // a truncated vertex is off by less (three components of 2^-20 X)
     for (int64_t m = (int64_t)atomicAdd(next, 1ull); m < M; m = (int64_t)atomicAdd(next, 1ull)) {
         const double px = S[3 * m], py = S[3 * m + 1], pz = S[3 * m + 2];
-        poly_box(P, box);
+        poly_box(P, C, box);
         // Float32 work that keeps most candidates off the float64 pipe, which a
         // warp pays for all its lanes whenever one of them uses it. Sites are
         // float32 values, so pf and the candidates are exact.
@@ -405,7 +412,7 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
         //    is dropped only beyond reach^2 (1 + 2^-17).
         //  * far vertices: a candidate at distance D can only cut vertices at
         //    least D/2 from the site, so with candidates taken nearest first a
-        //    shrinking list of vertices (W.far) has to be tested.
+        //    shrinking list of vertices (P.far) has to be tested.
         //  * screen: the candidate's plane n.v = n.p + |n|^2/2 (n not normalised)
         //    against those vertices. Truncation and rounding leave n.v and the
         //    right side within |n|_1 X 2^-19; a candidate is dropped when every
@@ -425,15 +432,15 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
             const float hm2 = __fmul_rd(hm, hm);
             float r2 = 0.f;
             nfar = 0;
-            for (int i = 0; i < P.nv; i++) {
-                const float vx = trunc_float(P.x[i]), vy = trunc_float(P.y[i]), vz = trunc_float(P.z[i]);
+            for (int i = 0; i < C.nv; i++) {
+                const float vx = trunc_float(P.v[i].x), vy = trunc_float(P.v[i].y), vz = trunc_float(P.v[i].z);
                 const float dx = vx - pf.x, dy = vy - pf.y, dz = vz - pf.z;
                 const float r = __fmaf_ru(dz, dz, __fmaf_ru(dy, dy, __fmul_ru(dx, dx)));
                 r2 = fmaxf(r2, r);
                 if (r >= hm2) {
-                    W.far[3 * nfar] = vx;
-                    W.far[3 * nfar + 1] = vy;
-                    W.far[3 * nfar + 2] = vz;
+                    P.far[3 * nfar] = vx;
+                    P.far[3 * nfar + 1] = vy;
+                    P.far[3 * nfar + 2] = vz;
                     nfar++;
                 }
             }
@@ -458,32 +465,30 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
         // bits), and the buffer becomes a binary min-heap when it is
         // drained, so each pick costs a walk down the heap rather than a
         // scan of the whole buffer.
-        constexpr int kBuf = 384;
-        unsigned long long bkey[kBuf];
         int nb = 0;
         auto sift_down = [&](int i, unsigned long long v) {
             for (;;) {
                 int c = 2 * i + 1;
                 if (c >= nb) break;
-                unsigned long long cv = bkey[c];
+                unsigned long long cv = P.key[c];
                 if (c + 1 < nb) {
-                    const unsigned long long c2 = bkey[c + 1];
+                    const unsigned long long c2 = P.key[c + 1];
                     if (c2 < cv) { cv = c2; c++; }
                 }
                 if (v <= cv) break;
-                bkey[i] = cv;
+                P.key[i] = cv;
                 i = c;
             }
-            bkey[i] = v;
+            P.key[i] = v;
         };
         auto flush = [&]() -> int {
             if (nb == 0) return 0;
-            for (int i = nb / 2 - 1; i >= 0; i--) sift_down(i, bkey[i]);
-            refresh(__uint_as_float((unsigned)(bkey[0] >> 32)));
+            for (int i = nb / 2 - 1; i >= 0; i--) sift_down(i, P.key[i]);
+            refresh(__uint_as_float((unsigned)(P.key[0] >> 32)));
             while (nb > 0) {
-                const unsigned long long top = bkey[0];
+                const unsigned long long top = P.key[0];
                 nb--;
-                if (nb > 0) sift_down(0, bkey[nb]);
+                if (nb > 0) sift_down(0, P.key[nb]);
                 const float d2k = __uint_as_float((unsigned)(top >> 32));
                 const int jj = (int)(unsigned)top;
                 if (d2k > R2f) {
@@ -498,8 +503,8 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
                     const float T = __fadd_rn(np, __fmaf_rn(0.5f, d2k, -n1 * Xf * 0x1p-18f));
                     bool maybe = false;
                     for (int i = 0; i < nfar && !maybe; i++) {
-                        const float v = __fmaf_rn(fz, W.far[3 * i + 2],
-                                                  __fmaf_rn(fy, W.far[3 * i + 1], __fmul_rn(fx, W.far[3 * i])));
+                        const float v = __fmaf_rn(fz, P.far[3 * i + 2],
+                                                  __fmaf_rn(fy, P.far[3 * i + 1], __fmul_rn(fx, P.far[3 * i])));
                         maybe = !(v <= T);
                     }
                     if (!maybe) continue;
@@ -509,7 +514,7 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
                 const double dist = sqrt(dx * dx + dy * dy + dz * dz);
                 const double nx = dx / dist, ny = dy / dist, nz = dz / dist;
                 const double d = nx * 0.5 * (qx + px) + ny * 0.5 * (qy + py) + nz * 0.5 * (qz + pz);
-                const int rc = poly_cut(P, W, nx, ny, nz, d, jj, eps);
+                const int rc = poly_cut(P, C, nx, ny, nz, d, jj, eps);
                 if (rc < 0) return 1;
                 if (rc > 0) refresh(d2k);
             }
@@ -537,7 +542,7 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
                             if (d2f > R2f) continue;
                             if (nb == kBuf) fail = flush();
                             if (fail) break;
-                            bkey[nb++] = ((unsigned long long)__float_as_uint(d2f) << 32) | (unsigned)jj;
+                            P.key[nb++] = ((unsigned long long)__float_as_uint(d2f) << 32) | (unsigned)jj;
                         }
                     }
                 }
@@ -557,39 +562,40 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
         }
         // faces of positive area -> neighbours; volume as pyramids from the site; bounding box
         static_assert(kNE >= kCap, "the edge keys hold the neighbour list");
-        int *const ids = W.ekey;  // free once the cuts are done
+        int *const ids = P.ekey;  // free once the cuts are done
         int cnt = 0;
         double vol = 0.0;
         double bb[6] = {1e300, 1e300, 1e300, -1e300, -1e300, -1e300};
-        for (int f = 0; f < P.nf && !fail; f++) {
-            const int b = P.fbeg[f], k = P.flen[f];
+        for (int f = 0; f < C.nf && !fail; f++) {
+            const Face fc = P.face[f];
+            const int b = fc.beg, k = fc.len;
             const int v0 = P.L[b];
             double sx = 0, sy = 0, sz = 0, sv = 0;
             for (int t = 1; t + 1 < k; t++) {
                 const int v1 = P.L[b + t], v2 = P.L[b + t + 1];
-                const double ax = P.x[v1] - P.x[v0], ay = P.y[v1] - P.y[v0], az = P.z[v1] - P.z[v0];
-                const double cx = P.x[v2] - P.x[v0], cy = P.y[v2] - P.y[v0], cz = P.z[v2] - P.z[v0];
+                const double ax = P.v[v1].x - P.v[v0].x, ay = P.v[v1].y - P.v[v0].y, az = P.v[v1].z - P.v[v0].z;
+                const double cx = P.v[v2].x - P.v[v0].x, cy = P.v[v2].y - P.v[v0].y, cz = P.v[v2].z - P.v[v0].z;
                 const double ux = ay * cz - az * cy, uy = az * cx - ax * cz, uz = ax * cy - ay * cx;
                 sx += ux;
                 sy += uy;
                 sz += uz;
                 // signed volume of the tetrahedron (site, v0, v1, v2)
-                sv += ((P.x[v0] - px) * ux + (P.y[v0] - py) * uy + (P.z[v0] - pz) * uz) / 6.0;
+                sv += ((P.v[v0].x - px) * ux + (P.v[v0].y - py) * uy + (P.v[v0].z - pz) * uz) / 6.0;
             }
             vol += fabs(sv);
             const double area2 = sx * sx + sy * sy + sz * sz;
             if (area2 > 0.0) {
                 if (cnt >= kCap) { fail = 1; break; }
-                ids[cnt++] = P.fid[f];
+                ids[cnt++] = fc.id;
             }
         }
-        for (int i = 0; i < P.nv; i++) {
-            bb[0] = fmin(bb[0], P.x[i]);
-            bb[1] = fmin(bb[1], P.y[i]);
-            bb[2] = fmin(bb[2], P.z[i]);
-            bb[3] = fmax(bb[3], P.x[i]);
-            bb[4] = fmax(bb[4], P.y[i]);
-            bb[5] = fmax(bb[5], P.z[i]);
+        for (int i = 0; i < C.nv; i++) {
+            bb[0] = fmin(bb[0], P.v[i].x);
+            bb[1] = fmin(bb[1], P.v[i].y);
+            bb[2] = fmin(bb[2], P.v[i].z);
+            bb[3] = fmax(bb[3], P.v[i].x);
+            bb[4] = fmax(bb[4], P.v[i].y);
+            bb[5] = fmax(bb[5], P.v[i].z);
         }
         // the list in ascending order without repeats (insertion sort: a few
         // dozen ids), as the host's CSR holds it
@@ -667,9 +673,10 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
     int *bidx = nullptr, *bsites = nullptr, *cnt = nullptr, *nbr = nullptr, *fail = nullptr;
     int64_t *boff = nullptr, *cursor = nullptr, *tmp = nullptr, *doff = nullptr;
     int *didx = nullptr;
+    Cell *pool = nullptr;
     double *vol = nullptr, *bbox = nullptr;
     auto cleanup = [&]() {
-        void *ptrs[] = {dS, dE, dSf, bidx, bsites, cnt, nbr, fail, boff, cursor, tmp, vol, bbox, doff, didx};
+        void *ptrs[] = {dS, dE, dSf, bidx, bsites, cnt, nbr, fail, boff, cursor, tmp, vol, bbox, doff, didx, pool};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     };
@@ -732,10 +739,16 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
     // take 2.3 ms instead of 6.1, 10^4 clumpy ones 8.2 instead of 14.6 (cell phase).
     const int lanes = (int)std::min<int64_t>(32, std::max<int64_t>(1, M / ((int64_t)sms * 32)));
     const int64_t per_block = 4 * lanes;
-    const int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((M + per_block - 1) / per_block, (int64_t)per_sm * sms));
+    int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((M + per_block - 1) / per_block, (int64_t)per_sm * sms));
     if ((e = cudaMemset(cursor, 0, sizeof(unsigned long long))) != cudaSuccess) return bad(e, "memset");
+    // 1.5 GB for a GPU full of threads; with less room, fewer threads take turns
+    while ((e = cudaMalloc(&pool, sizeof(Cell) * cblocks * per_block)) != cudaSuccess) {
+        if (cblocks == 1) return bad(e, "alloc");
+        cudaGetLastError();
+        cblocks /= 2;
+    }
     cells_kernel<<<cblocks, 128>>>(dS, M, bg, boff, bsites, box[0], box[1], box[2], box[3], box[4], box[5], eps, cnt,
-                                   nbr, vol, bbox, fail, reinterpret_cast<unsigned long long *>(cursor), dSf, lanes);
+                                   nbr, vol, bbox, fail, reinterpret_cast<unsigned long long *>(cursor), dSf, lanes, pool);
     count_launches(6);  // keys, grid lines, bucket count, fill, sort, cells (the scan counts its own)
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bad(e, "cells kernel");
     std::vector<int> hcnt(M), hfail(M);
