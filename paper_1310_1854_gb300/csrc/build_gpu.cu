@@ -208,6 +208,20 @@ __global__ void bucket_sort_kernel(const int64_t *off, int64_t K, int *bsites) {
     }
 }
 
+// The sites in bucket order, each with its index: the buckets of a row are one run
+// of 16-byte entries, read four at a time. Before, each bucket's bounds, its
+// sites' indices and their positions were three dependent reads one after the
+// other, and every bucket of a ring was visited; rows and slabs of buckets out of
+// reach are skipped now. The longest search binds a small grid: cell phase at
+// 10^5 disk sites 32.4 -> 21.6 ms.
+__global__ void bucket_sites_kernel(const float4 *Sf, const int *bsites, int64_t M, float4 *Sb) {
+    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < M; q += (int64_t)gridDim.x * blockDim.x) {
+        const int m = bsites[q];
+        const float4 p = __ldg(Sf + m);
+        Sb[q] = make_float4(p.x, p.y, p.z, __int_as_float(m));
+    }
+}
+
 // counts of the polyhedron, in registers
 struct Counts {
     int nv, nf, nl;
@@ -384,10 +398,10 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
 // as it has finished one, so a thread whose cell needed few cuts does not
 // wait for the slowest cell of its block. Eight blocks of 128 per SM (64
 // registers): the kernel waits on its polyhedra and gains more from the extra
-// warps than it loses to the spills where cells are many (10^6 clumpy sites: 105 ms, 111 with six
-// blocks, 117 with five; 10^5: 20.9, 19.4 and 19.3).
+// warps than it loses to the spills where cells are many (10^6 clumpy sites: 103 ms, 109 with six
+// blocks, 114 with five; 10^5: 20.8, 19.8 and 18.9).
 __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t M, BucketGrid bg, const int64_t *boff,
-                                                    const int *bsites, double box0, double box1, double box2,
+                                                    const float4 *Sb, double box0, double box1, double box2,
                                                     double box3, double box4, double box5, double eps, int *out_cnt,
                                                     int *out_nbr, double *out_vol, double *out_bbox, int *out_fail,
                                                     unsigned long long *next, const float4 *Sf, int lanes,
@@ -520,30 +534,50 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
             }
             return 0;
         };
+        // one run of the sites in bucket order: those within reach go into the buffer
+        auto scan = [&](int64_t q, int64_t end) -> int {
+            for (; q < end; q += 4) {
+                float4 c[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) c[u] = __ldg(Sb + min(q + u, end - 1));
+#pragma unroll
+                for (int u = 0; u < 4; u++) {
+                    const float fx = __fsub_rn(c[u].x, pf.x), fy = __fsub_rn(c[u].y, pf.y), fz = __fsub_rn(c[u].z, pf.z);
+                    const float d2f = __fmaf_rn(fz, fz, __fmaf_rn(fy, fy, __fmul_rn(fx, fx)));
+                    const int jj = __float_as_int(c[u].w);
+                    if (q + u >= end || d2f > R2f || jj == (int)m) continue;
+                    if (nb == kBuf && flush()) return 1;
+                    P.key[nb++] = ((unsigned long long)__float_as_uint(d2f) << 32) | (unsigned)jj;
+                }
+            }
+            return 0;
+        };
+        // Distance along one axis from the site to the sites of bucket i (edge[i] <= v
+        // <= edge[i + 1]), rounded down. A slab or row of buckets is skipped where it
+        // takes every site beyond reach by more than the rounding of d2f (2^-21).
+        auto off_axis = [&](int c, int i) {
+            const double *e = bg.edge[c] + i;
+            return __double2float_rd(fmax(fmax(__ldg(e) - pc[c], pc[c] - __ldg(e + 1)), 0.0));
+        };
         for (int s = 0; s <= smax && !fail; s++) {
-            for (int di = -s; di <= s && !fail; di++) {
-                const int i = bi + di;
-                if (i < 0 || i >= bg.dim[0]) continue;
-                for (int dj = -s; dj <= s && !fail; dj++) {
-                    const int j = bj + dj;
-                    if (j < 0 || j >= bg.dim[1]) continue;
-                    const bool shell = abs(di) == s || abs(dj) == s;
-                    for (int dk = -s; dk <= s && !fail; dk += (shell || s == 0) ? 1 : 2 * s) {
-                        const int k = bk + dk;
-                        if (k < 0 || k >= bg.dim[2]) continue;
-                        const int b = (i * bg.dim[1] + j) * bg.dim[2] + k;
-                        for (int64_t q = boff[b]; q < boff[b + 1]; q++) {
-                            const int jj = bsites[q];
-                            if (jj == (int)m) continue;
-                            const float4 qf = Sf[jj];
-                            const float fx = __fsub_rn(qf.x, pf.x), fy = __fsub_rn(qf.y, pf.y),
-                                        fz = __fsub_rn(qf.z, pf.z);
-                            const float d2f = __fmaf_rn(fz, fz, __fmaf_rn(fy, fy, __fmul_rn(fx, fx)));
-                            if (d2f > R2f) continue;
-                            if (nb == kBuf) fail = flush();
-                            if (fail) break;
-                            P.key[nb++] = ((unsigned long long)__float_as_uint(d2f) << 32) | (unsigned)jj;
+            for (int i = max(bi - s, 0); i <= min(bi + s, bg.dim[0] - 1) && !fail; i++) {
+                const float ox = off_axis(0, i), ox2 = __fmul_rd(ox, ox);
+                if (ox2 * (1.0f - 0x1p-19f) > R2f) continue;
+                for (int j = max(bj - s, 0); j <= min(bj + s, bg.dim[1] - 1) && !fail; j++) {
+                    const float oy = off_axis(1, j);
+                    if (__fmaf_rd(oy, oy, ox2) * (1.0f - 0x1p-19f) > R2f) continue;
+                    const int64_t *row = boff + (int64_t)(i * bg.dim[1] + j) * bg.dim[2];
+                    // a row of the shell is one run; inside the shell its two ends are
+                    const bool shell = abs(i - bi) == s || abs(j - bj) == s;
+                    for (int r = 0; r < (shell ? 1 : 2) && !fail; r++) {
+                        int k0 = r == 0 ? bk - s : bk + s, k1 = shell ? bk + s : k0;
+                        if (shell) {
+                            k0 = max(k0, 0);
+                            k1 = min(k1, bg.dim[2] - 1);
+                        } else if (k0 < 0 || k0 >= bg.dim[2]) {
+                            continue;
                         }
+                        fail = scan(__ldg(row + k0), __ldg(row + k1 + 1));
                     }
                 }
             }
@@ -669,14 +703,14 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         lines += bg.dim[c] + 1;
     }
     double *dS = nullptr, *dE = nullptr;
-    float4 *dSf = nullptr;
+    float4 *dSf = nullptr, *dSb = nullptr;
     int *bidx = nullptr, *bsites = nullptr, *cnt = nullptr, *nbr = nullptr, *fail = nullptr;
     int64_t *boff = nullptr, *cursor = nullptr, *tmp = nullptr, *doff = nullptr;
     int *didx = nullptr;
     Cell *pool = nullptr;
     double *vol = nullptr, *bbox = nullptr;
     auto cleanup = [&]() {
-        void *ptrs[] = {dS, dE, dSf, bidx, bsites, cnt, nbr, fail, boff, cursor, tmp, vol, bbox, doff, didx, pool};
+        void *ptrs[] = {dS, dE, dSf, dSb, bidx, bsites, cnt, nbr, fail, boff, cursor, tmp, vol, bbox, doff, didx, pool};
         for (void *p : ptrs)
             if (p) cudaFree(p);
     };
@@ -708,6 +742,7 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         for (int64_t m = 0; m < M; m++)
             sf[m] = make_float4((float)S[3 * m], (float)S[3 * m + 1], (float)S[3 * m + 2], 0.f);
         if ((e = cudaMalloc(&dSf, sizeof(float4) * M)) != cudaSuccess) return bad(e, "alloc");
+        if ((e = cudaMalloc(&dSb, sizeof(float4) * M)) != cudaSuccess) return bad(e, "alloc");
         if ((e = cudaMemcpy(dSf, sf.data(), sizeof(float4) * M, cudaMemcpyHostToDevice)) != cudaSuccess)
             return bad(e, "upload");
     }
@@ -729,6 +764,7 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         return bad(e, "copy");
     bucket_fill_kernel<<<blocks, 256>>>(bidx, M, cursor, bsites);
     bucket_sort_kernel<<<(int)std::min<int64_t>((K + 255) / 256, 65535), 256>>>(boff, K, bsites);
+    bucket_sites_kernel<<<blocks, 256>>>(dSf, bsites, M, dSb);
     int dev = 0, sms = 1, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -747,9 +783,9 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         cudaGetLastError();
         cblocks /= 2;
     }
-    cells_kernel<<<cblocks, 128>>>(dS, M, bg, boff, bsites, box[0], box[1], box[2], box[3], box[4], box[5], eps, cnt,
+    cells_kernel<<<cblocks, 128>>>(dS, M, bg, boff, dSb, box[0], box[1], box[2], box[3], box[4], box[5], eps, cnt,
                                    nbr, vol, bbox, fail, reinterpret_cast<unsigned long long *>(cursor), dSf, lanes, pool);
-    count_launches(6);  // keys, grid lines, bucket count, fill, sort, cells (the scan counts its own)
+    count_launches(7);  // keys, grid lines, bucket count, fill, sort, sites, cells (the scan counts its own)
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bad(e, "cells kernel");
     std::vector<int> hcnt(M), hfail(M);
     out.vol.assign(M, 0.0);
