@@ -58,20 +58,13 @@ struct Cell {
         double x, y, z, f;  // f: the value of the cutting plane
     } v[kNV];
     Face face[kNF];
-    unsigned char L[kNL];
+    unsigned char L[2][kNL];       // face loops: the current ones and those a cut writes
     unsigned long long key[kBuf];  // candidates: distance bits above the site
+    float far[3 * kNV];            // the vertices a candidate can still cut
+    unsigned char rank[kNV];       // order of the vertices
     // scratch of a cut
-    union {
-        struct {
-            double x, y, z;
-        } w[kNV];              // the vertices kept by a cut
-        float far[3 * kNV];    // between cuts: the vertices a candidate can still cut
-    };
-    Face face2[kNF];
-    unsigned char L2[kNL];
     int ekey[kNE];
     unsigned char evid[kNE];
-    unsigned char remap[kNV];
     unsigned char seg_a[kNF], seg_b[kNF];
 };
 static_assert(sizeof(Cell) % 32 == 0, "every cell starts on a sector");
@@ -222,14 +215,28 @@ __global__ void bucket_sites_kernel(const float4 *Sf, const int *bsites, int64_t
     }
 }
 
-// counts of the polyhedron, in registers
+// What a thread keeps of its polyhedron in registers. A vertex stays where it
+// was made until a cut drops it, and new ones take the lowest free places; the
+// order of the vertices, which decides the end that a new vertex is formed from,
+// is a byte of its own, and the loops alternate between two arrays. Before, each
+// cut renumbered the vertices, copied them to scratch and back and rewrote the
+// loops: cell phase at 10^6 clumpy sites 103 -> 98 ms, 3 10^5 uniform ones 30.5 ->
+// 28.7, at 10^5 the same within 1 %.
 struct Counts {
-    int nv, nf, nl;
+    unsigned long long use0, use1;  // places taken
+    int end;                        // places past the last one taken
+    int nf, cur;                    // faces, and which loops are current
 };
+__device__ __forceinline__ bool bit128(unsigned long long m0, unsigned long long m1, int v) {
+    return ((v < 64 ? m0 >> v : m1 >> (v - 64)) & 1ull) != 0ull;
+}
 
 __device__ void poly_box(Cell &P, Counts &C, const double *box) {
-    C.nv = 8;
+    C.use0 = 0xffull;
+    C.use1 = 0ull;
+    C.end = 8;
     for (int i = 0; i < 8; i++) {
+        P.rank[i] = (unsigned char)i;
         P.v[i].x = (i & 4) ? box[3] : box[0];
         P.v[i].y = (i & 2) ? box[4] : box[1];
         P.v[i].z = (i & 1) ? box[5] : box[2];
@@ -237,10 +244,10 @@ __device__ void poly_box(Cell &P, Counts &C, const double *box) {
     // counter-clockwise seen from outside; walls -1..-6 = x min, x max, y min, y max, z min, z max
     const unsigned char quad[6][4] = {{0, 1, 3, 2}, {4, 6, 7, 5}, {0, 4, 5, 1}, {2, 3, 7, 6}, {0, 2, 6, 4}, {1, 5, 7, 3}};
     C.nf = 6;
-    C.nl = 24;
+    C.cur = 0;
     for (int w = 0; w < 6; w++) {
         P.face[w] = Face{-(w + 1), (short)(4 * w), 4};
-        for (int k = 0; k < 4; k++) P.L[4 * w + k] = quad[w][k];
+        for (int k = 0; k < 4; k++) P.L[0][4 * w + k] = quad[w][k];
     }
 }
 
@@ -264,7 +271,8 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
     static_assert(kNV <= 128, "vertex masks hold 128 bits");
     unsigned long long out0 = 0ull, out1 = 0ull, str0 = 0ull, str1 = 0ull;
     const long long eb = __double_as_longlong(eps);
-    for (int i = 0; i < C.nv; i++) {
+    for (int i = 0; i < C.end; i++) {
+        if (!bit128(C.use0, C.use1, i)) continue;
         const double f = nx * P.v[i].x + ny * P.v[i].y + nz * P.v[i].z - d;
         P.v[i].f = f;
         const long long fb = __double_as_longlong(f);
@@ -280,50 +288,56 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
         }
     }
     if (!(out0 | out1)) return 0;
-    auto is_out = [&](int v) { return ((v < 64 ? out0 >> v : out1 >> (v - 64)) & 1ull) != 0ull; };
-    auto is_strict = [&](int v) { return ((v < 64 ? str0 >> v : str1 >> (v - 64)) & 1ull) != 0ull; };
-    int ne = 0, nseg = 0, nf2 = 0, nl2 = 0, nv = C.nv;
+    auto is_out = [&](int v) { return bit128(out0, out1, v); };
+    auto is_strict = [&](int v) { return bit128(str0, str1, v); };
+    const unsigned char *const L = P.L[C.cur];
+    unsigned char *const L2 = P.L[C.cur ^ 1];
+    unsigned long long free0 = ~C.use0, free1 = ~C.use1 & ((1ull << (kNV - 64)) - 1ull);
+    int ne = 0, nseg = 0, nf2 = 0, nl2 = 0;
     for (int f = 0; f < C.nf; f++) {
         const Face fc = P.face[f];
         const int b = fc.beg, k = fc.len;
         const int start = nl2;
         int entry = -1, exit_ = -1;
         // one pass: a face wholly above the plane leaves no entries
-        int vb = P.L[b];
+        int vb = L[b];
         bool bo = is_out(vb);
         for (int i = 1; i <= k; i++) {
             const int va = vb;
             const bool ao = bo;
-            vb = P.L[b + (i < k ? i : 0)];
+            vb = L[b + (i < k ? i : 0)];
             bo = is_out(vb);
             if (!ao) {
                 if (nl2 >= kNL) return -1;
-                P.L2[nl2++] = (unsigned char)va;
+                L2[nl2++] = (unsigned char)va;
             }
             if (ao != bo) {
                 const bool strict = !ao ? is_strict(va) : is_strict(vb);
                 int x = !ao ? va : vb;
                 if (strict) {
                     // the vertex on edge (va, vb), made once from the lower index
-                    const int lo = min(va, vb), hi = max(va, vb);
+                    const bool up = P.rank[va] < P.rank[vb];
+                    const int lo = up ? va : vb, hi = up ? vb : va;
                     const int key = lo * 256 + hi;
                     x = -1;
                     for (int e = 0; e < ne; e++)
                         if (P.ekey[e] == key) { x = P.evid[e]; break; }
                     if (x < 0) {
-                        if (ne >= kNE || nv >= kNV) return -1;
+                        if (ne >= kNE || !(free0 | free1)) return -1;
+                        x = free0 ? __ffsll((long long)free0) - 1 : 63 + __ffsll((long long)free1);
+                        if (free0) free0 &= free0 - 1;
+                        else free1 &= free1 - 1;
                         const auto vl = P.v[lo], vh = P.v[hi];
                         const double t = vl.f / (vl.f - vh.f);
-                        P.v[nv].x = vl.x + t * (vh.x - vl.x);
-                        P.v[nv].y = vl.y + t * (vh.y - vl.y);
-                        P.v[nv].z = vl.z + t * (vh.z - vl.z);
+                        P.v[x].x = vl.x + t * (vh.x - vl.x);
+                        P.v[x].y = vl.y + t * (vh.y - vl.y);
+                        P.v[x].z = vl.z + t * (vh.z - vl.z);
                         P.ekey[ne] = key;
-                        P.evid[ne] = (unsigned char)nv;
+                        P.evid[ne] = (unsigned char)x;
                         ne++;
-                        x = nv++;
                     }
                     if (nl2 >= kNL) return -1;
-                    P.L2[nl2++] = (unsigned char)x;
+                    L2[nl2++] = (unsigned char)x;
                 }
                 if (!ao) exit_ = x;
                 else entry = x;
@@ -337,7 +351,7 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
         }
         if (nl2 > start && nf2 >= kNF) return -1;
         if (nl2 - start >= 3) {
-            P.face2[nf2++] = Face{fc.id, (short)start, (short)(nl2 - start)};
+            P.face[nf2++] = Face{fc.id, (short)start, (short)(nl2 - start)};
         } else {
             nl2 = start;
         }
@@ -356,41 +370,32 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
             if (pick < 0) { ok = false; break; }
             used |= 1ull << pick;
             if (nl2 >= kNL) return -1;
-            P.L2[nl2++] = P.seg_a[pick];
+            L2[nl2++] = P.seg_a[pick];
             cur = P.seg_b[pick];
         }
         if (!ok || cur != first) return -1;  // inconsistent topology: leave it to the host
         if (nl2 - start >= 3) {
             if (nf2 >= kNF) return -1;
-            P.face2[nf2++] = Face{id, (short)start, (short)(nl2 - start)};
+            P.face[nf2++] = Face{id, (short)start, (short)(nl2 - start)};
         } else {
             nl2 = start;
         }
     }
-    // compact the vertices that are still referenced
-    for (int i = 0; i < nv; i++) P.remap[i] = 255;
-    int nv2 = 0;
+    // the vertices still referenced, ranked by their first place in the loops
+    unsigned long long met0 = 0ull, met1 = 0ull;
+    int n = 0;
     for (int i = 0; i < nl2; i++) {
-        const int v = P.L2[i];
-        int r = P.remap[v];
-        if (r == 255) {
-            r = nv2++;
-            P.remap[v] = (unsigned char)r;
-            P.w[r].x = P.v[v].x;
-            P.w[r].y = P.v[v].y;
-            P.w[r].z = P.v[v].z;
-        }
-        P.L[i] = (unsigned char)r;
+        const int v = L2[i];
+        if (bit128(met0, met1, v)) continue;
+        if (v < 64) met0 |= 1ull << v;
+        else met1 |= 1ull << (v - 64);
+        P.rank[v] = (unsigned char)n++;
     }
-    for (int i = 0; i < nv2; i++) {
-        P.v[i].x = P.w[i].x;
-        P.v[i].y = P.w[i].y;
-        P.v[i].z = P.w[i].z;
-    }
-    C.nv = nv2;
-    C.nl = nl2;
+    C.use0 = met0;
+    C.use1 = met1;
+    C.end = met1 ? 128 - __clzll((long long)met1) : 64 - __clzll((long long)met0);
+    C.cur ^= 1;
     C.nf = nf2;
-    for (int f = 0; f < nf2; f++) P.face[f] = P.face2[f];
     return nf2 >= 4 ? 1 : -1;
 }
 
@@ -398,8 +403,10 @@ __device__ int poly_cut(Cell &P, Counts &C, double nx, double ny, double nz, dou
 // as it has finished one, so a thread whose cell needed few cuts does not
 // wait for the slowest cell of its block. Eight blocks of 128 per SM (64
 // registers): the kernel waits on its polyhedra and gains more from the extra
-// warps than it loses to the spills where cells are many (10^6 clumpy sites: 103 ms, 109 with six
-// blocks, 114 with five; 10^5: 20.8, 19.8 and 18.9).
+// warps than it loses to the spills where cells are many (cell phase at 10^6
+// clumpy sites: 98 ms, 101 with six blocks, 106 with five; 10^5 clumpy: 20.8, 18.7
+// and 18.5, but 10^5 disk sites 21.7, 22.9 and 22.5 and 10^4 clumpy 4.82, 5.01 and
+// 5.03).
 __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t M, BucketGrid bg, const int64_t *boff,
                                                     const float4 *Sb, double box0, double box1, double box2,
                                                     double box3, double box4, double box5, double eps, int *out_cnt,
@@ -446,7 +453,8 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
             const float hm2 = __fmul_rd(hm, hm);
             float r2 = 0.f;
             nfar = 0;
-            for (int i = 0; i < C.nv; i++) {
+            for (int i = 0; i < C.end; i++) {
+                if (!bit128(C.use0, C.use1, i)) continue;
                 const float vx = trunc_float(P.v[i].x), vy = trunc_float(P.v[i].y), vz = trunc_float(P.v[i].z);
                 const float dx = vx - pf.x, dy = vy - pf.y, dz = vz - pf.z;
                 const float r = __fmaf_ru(dz, dz, __fmaf_ru(dy, dy, __fmul_ru(dx, dx)));
@@ -600,13 +608,14 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
         int cnt = 0;
         double vol = 0.0;
         double bb[6] = {1e300, 1e300, 1e300, -1e300, -1e300, -1e300};
+        const unsigned char *const L = P.L[C.cur];
         for (int f = 0; f < C.nf && !fail; f++) {
             const Face fc = P.face[f];
             const int b = fc.beg, k = fc.len;
-            const int v0 = P.L[b];
+            const int v0 = L[b];
             double sx = 0, sy = 0, sz = 0, sv = 0;
             for (int t = 1; t + 1 < k; t++) {
-                const int v1 = P.L[b + t], v2 = P.L[b + t + 1];
+                const int v1 = L[b + t], v2 = L[b + t + 1];
                 const double ax = P.v[v1].x - P.v[v0].x, ay = P.v[v1].y - P.v[v0].y, az = P.v[v1].z - P.v[v0].z;
                 const double cx = P.v[v2].x - P.v[v0].x, cy = P.v[v2].y - P.v[v0].y, cz = P.v[v2].z - P.v[v0].z;
                 const double ux = ay * cz - az * cy, uy = az * cx - ax * cz, uz = ax * cy - ay * cx;
@@ -623,7 +632,8 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
                 ids[cnt++] = fc.id;
             }
         }
-        for (int i = 0; i < C.nv; i++) {
+        for (int i = 0; i < C.end; i++) {
+            if (!bit128(C.use0, C.use1, i)) continue;
             bb[0] = fmin(bb[0], P.v[i].x);
             bb[1] = fmin(bb[1], P.v[i].y);
             bb[2] = fmin(bb[2], P.v[i].z);
