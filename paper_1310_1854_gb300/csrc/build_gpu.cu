@@ -51,7 +51,7 @@ constexpr int kBuf = 384;  // candidates of one drain
 // A thread's polyhedron and scratch: a run of global memory of its own. Local
 // memory deals the threads' 4-byte words out in turn, so with the lanes of a warp
 // at different cells (about 4 of 32 run together) every access moved a 32-byte
-// sector for 4 bytes of it: 80 GB of DRAM traffic for 2 10^5 clumpy cells, 24 now,
+// sector for 4 bytes of it: 80 GB of DRAM traffic for 2 10^5 clumpy cells, 18 now,
 // L1 hits 46 -> 81 %. Cell kernel 23.6 -> 15.8 ms at 10^5 clumpy sites, cell phase
 // 138 -> 107 ms at 10^6. (32-byte vertices moved as pairs of double2: 2 % slower.)
 struct Cell {
@@ -799,7 +799,7 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
     const int64_t per_block = 4 * lanes;
     int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((M + per_block - 1) / per_block, (int64_t)per_sm * sms));
     if ((e = cudaMemset(cursor, 0, sizeof(unsigned long long))) != cudaSuccess) return bad(e, "memset");
-    // 1.5 GB for a GPU full of threads; with less room, fewer threads take turns
+    // 1.4 GB for a GPU full of threads; with less room, fewer threads take turns
     while ((e = cudaMalloc(&pool, sizeof(Cell) * cblocks * per_block)) != cudaSuccess) {
         if (cblocks == 1) return bad(e, "alloc");
         cudaGetLastError();
