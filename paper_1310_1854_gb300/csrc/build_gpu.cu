@@ -450,7 +450,8 @@ __global__ void __launch_bounds__(128, 8) cells_kernel(const double *S, int64_t 
         // the largest radius taken in float64 after each cut: 30,000 sites in a
         // ball, whose surface cells reach the corners of the box and meet tens of
         // thousands of candidates, took 409 ms instead of 137, 10^5 disk sites 55
-        // instead of 52, 10^6 clumpy ones 159 instead of 144 (cell phase).
+        // instead of 52, 10^6 clumpy ones 159 instead of 144 (cell phase, with the
+        // polyhedra still in local memory; the last two take 21 and 97 ms now).
         const float4 pf = Sf[m];
         float R2f = 0.f, reach = 0.f;
         int nfar = 0;
@@ -794,7 +795,8 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
         per_sm = 1;
     // The lanes of a warp take turns wherever their cells differ, so few cells
     // are spread over all warps that fit, down to one cell per warp: 1000 cells
-    // take 2.3 ms instead of 6.1, 10^4 clumpy ones 8.2 instead of 14.6 (cell phase).
+    // take 2.3 ms instead of 6.1, 10^4 clumpy ones 8.2 instead of 14.6 (cell phase,
+    // with the polyhedra still in local memory; 10^4 take 4.7 now).
     const int lanes = (int)std::min<int64_t>(32, std::max<int64_t>(1, M / ((int64_t)sms * 32)));
     const int64_t per_block = 4 * lanes;
     int cblocks = (int)std::max<int64_t>(1, std::min<int64_t>((M + per_block - 1) / per_block, (int64_t)per_sm * sms));
