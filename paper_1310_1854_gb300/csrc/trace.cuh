@@ -915,6 +915,9 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
         if (needmask) {
             int head = q_pos[0], cnt = q_pos[1];
             if (head == cnt) {
+                // other lanes read their slots in the last turn, and neither the
+                // ballot above nor the shuffle below orders memory
+                __syncwarp();
                 // refill: 32 rays while many are left, fewer towards the end (an
                 // eighth of what each warp of the launch has still to trace)
                 // so that no warp sits on rays that another could start, at
