@@ -15,6 +15,7 @@
 #include <mutex>
 #include <string>
 #include <tuple>
+#include <utility>
 #include <vector>
 
 #include "fsplit.h"
@@ -359,18 +360,23 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         return fail(o.gpu_build ? VGRID_ERR_CUDA : VGRID_ERR_BUILD, err);
     }
     lap(2, t_lap);
-    // device buffers that the cell construction left, freed on every way out
-    struct CellsGuard {
-        vg::CellsOut &c;
-        ~CellsGuard() {
-            if (c.d_off) cudaFree(c.d_off);
-            if (c.d_idx) cudaFree(c.d_idx);
-            if (c.d_bbox) cudaFree(c.d_bbox);
-            c.d_off = nullptr;
-            c.d_idx = nullptr;
-            c.d_bbox = nullptr;
+    // device buffers that the cell construction left, owned here (not by g, which
+    // the failing ways out delete first) and freed on every way out
+    struct DeviceCells {
+        int64_t *off;
+        int32_t *idx;
+        double *bbox;
+        void release() {
+            if (off) cudaFree(off);
+            if (idx) cudaFree(idx);
+            if (bbox) cudaFree(bbox);
+            off = nullptr;
+            idx = nullptr;
+            bbox = nullptr;
         }
-    };
+        ~DeviceCells() { release(); }
+    } left{std::exchange(g->cells.d_off, nullptr), std::exchange(g->cells.d_idx, nullptr),
+           std::exchange(g->cells.d_bbox, nullptr)};
     if (o.host_only) {
         vg::build_blocks(bbox, g->cells.bbox, M, o.blocks_per_site, g->blocks, o.threads);
         lap(3, t_lap);
@@ -417,7 +423,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         for (int c = 0; c < 3; c++) ddim[c] = (int32_t)std::min<long>(std::max<long>(std::lround(ext[c] / cs), 1), 256);
     }
     {
-        CellsGuard guard{g->cells};
         std::vector<float4> site4(M);
         vg::parallel_for(M, o.threads, 1 << 14, [&](int64_t i0, int64_t i1) {
             for (int64_t i = i0; i < i1; i++)
@@ -425,7 +430,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         });
         vg::block_dims(bbox, M, o.blocks_per_site, g->blocks.dim);
         vg::LayoutIn in{M, g->sms, bbox, {}, {}, site4.data(), g->perm.data(), g->cells.off.data(), g->cells.idx.data(),
-                        g->cells.bbox.data(), g->cells.d_off, g->cells.d_idx, g->cells.d_bbox};
+                        g->cells.bbox.data(), left.off, left.idx, left.bbox};
         for (int c = 0; c < 3; c++) {
             in.bdim[c] = g->blocks.dim[c];
             in.ddim[c] = ddim[c];
@@ -452,6 +457,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         g->phase_seconds[3] = lay.seconds[1];
         g->phase_seconds[4] = lay.seconds[2];
         g->phase_seconds[5] = lay.seconds[0];
+        left.release();
     }
     int rc = VGRID_OK;
 #define VG_ALLOC(p, n)                                              \
