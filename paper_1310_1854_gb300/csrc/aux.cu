@@ -127,7 +127,16 @@ __global__ void __launch_bounds__(256, PREP == PREP_CELL32 || PREP == PREP_CELL6
             two_sum(q1, q2, h, l);
             if (fp64) {
                 const float off = __fmaf_ru(kU, fabsf(h), __fmul_ru(0x1p-36f * scale, __fdiv_ru(1.0f, fabsf(kh))));
-                const float lo = __fsub_rd(h, off), hi = __fadd_ru(h, off);
+                float lo = __fsub_rd(h, off), hi = __fadd_ru(h, off);
+                if (!(off < __int_as_float(0x7f800000))) {
+                    // k_c is 0 in float32, or so small that the quotient is not a
+                    // finite number: no upper bound, and a lower one only where the
+                    // moved point is certainly off the wall (then |n| / |k_c|, with
+                    // |k_c| below |k_hi| (1 + 2^-22) + 2^-149)
+                    const float d = __fsub_rd(__fmul_rd(fabsf(nh), 1.0f - 0x1p-23f), 0x1p-36f * scale);
+                    hi = __int_as_float(0x7f800000);
+                    lo = d > 0.0f ? __fdiv_rd(d, __fadd_ru(__fmul_ru(fabsf(kh), 1.0f + 0x1p-22f), 0x1p-149f)) : -hi;
+                }
                 if (lo < w_lo) {
                     w_lo2 = w_lo;
                     w_lo = lo;
