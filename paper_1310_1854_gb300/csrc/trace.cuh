@@ -1293,9 +1293,12 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
         }
         if (FP64 && found) {
             // tau and the point for every lane before the paths part (a step of
-            // zero length adds zero to both): the float64 pipe bounds this form,
-            // and the lanes whose ray ends would run these again on their own
-            tau64 = __dadd_rn(tau64, __dmul_rn(__dmul_rn(fexact(kappa), fexact(rho)), s64));
+            // zero length adds zero to both, also where the density is infinite or
+            // NaN: the term is replaced, not the branch taken): the float64 pipe
+            // bounds this form, and the lanes whose ray ends would run these again
+            // on their own
+            const double term = __dmul_rn(__dmul_rn(fexact(kappa), fexact(rho)), s64);
+            tau64 = __dadd_rn(tau64, (int64_t)dbits(s64) > 0 ? term : 0.0);
             for (int c = 0; c < 3; c++) r64[c] = __dadd_rn(r64[c], __dmul_rn(s64, k64[c]));
             gone = __fadd_rn(gone, dtrunc(s64));
         }

@@ -74,3 +74,32 @@ def test_a_wall_at_zero(lanes):
         rc, rl = ref.segments(k)
         assert np.array_equal(sc[so[k]:so[k + 1]], rc), k
         assert np.all(np.abs(sl[so[k]:so[k + 1]] - rl) <= np.where(rl < 1e-6, 1e-12, 1e-12 * rl)), k
+
+
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_a_step_of_no_length_adds_nothing(bad):
+    """Rays that start on a face take a step of zero length through the cell
+    behind it, whatever that cell's density is."""
+    from paper_1310_1854_gb300 import VoronoiGrid
+    S = np.stack(np.meshgrid(*[np.arange(-0.75, 1.0, 0.5)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    rng = gen.rng_for(94)
+    rho = rng.uniform(0.5, 2.0, len(S)).astype(np.float32)
+    rho[rng.random(len(S)) < 0.3] = bad
+    n = 4000
+    o, d = gen.uniform_points(n, rng), gen.isotropic_dirs(n, rng)
+    i, ax = np.arange(n), rng.integers(0, 3, n)
+    o[i, ax] = rng.choice([-0.5, 0.0, 0.5], n)
+    vg = VoronoiGrid(S, gen.CUBE_BOX)
+    vg.set_density(dev(rho))
+    r = vg.trace(dev(o), dev(d), precision="fp64", segments=True, stats=True)
+    assert r.stats["zero_steps"] > n // 4
+    so, sc, sl = _segments(r)
+    want = np.array([np.sum(rho[sc[a:b]].astype(np.float64) * sl[a:b]) for a, b in zip(so[:-1], so[1:])])
+    for lanes in (1, 4):
+        vg.set_launch(fp64_lanes_per_ray=lanes)
+        for tau in (r.tau, vg.trace(dev(o), dev(d), precision="fp64").tau):
+            t = tau.cpu().numpy()
+            fine = np.isfinite(want)
+            assert fine.sum() > n // 50
+            np.testing.assert_allclose(t[fine], want[fine], rtol=1e-12)
+            assert np.array_equal(np.isnan(t), np.isnan(want)) and np.array_equal(np.isinf(t), np.isinf(want))
