@@ -169,10 +169,13 @@ typedef struct {
 
 /* launch shape of the traversal kernels */
 typedef struct {
-    int32_t lanes_per_ray;      /* 1, 2, 4 or 8 lanes cooperate on one ray (default 1) */
+    int32_t lanes_per_ray;      /* 2, 4 or 8: so many lanes cooperate on one ray. 1 (default):
+                                   one, or more in calls with too few rays to fill the GPU
+                                   that way; with blocks_per_sm > 0 always one */
     int32_t block;              /* threads per block (multiple of 32, 32..256; default 128) */
     int32_t blocks_per_sm;      /* persistent blocks per SM; 0 = as many as fit */
-    int32_t fp64_lanes_per_ray; /* lanes per ray of the float64 form; 0 = lanes_per_ray (default 1) */
+    int32_t fp64_lanes_per_ray; /* the same for the float64 form; 0 = lanes_per_ray (default 1).
+                                   Where it chooses, blocks of 128 may become smaller ones */
     int32_t order;              /* order in which the traversal takes the rays:
                                    1 = longest estimated path first (crossings estimated
                                    from a coarse site-density grid along each ray),
@@ -381,10 +384,9 @@ int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t 
                    const float *weight, int32_t *cell, float *s, float *absorbed, vgrid_stream_t stream);
 
 /* Launch shape used by this grid's traversal kernels. NULL resets to the
- * built-in default, which a new grid has: the shape that vgrid_get_launch
- * returns, except that calls with too few rays to fill the GPU at one lane per
- * ray use more lanes per ray (and smaller blocks in the float64 form). Results
- * do not depend on the shape. */
+ * built-in default, which a new grid has (1, 128, 0, 1, 0). Setting the shape
+ * that vgrid_get_launch returned changes nothing. Results do not depend on the
+ * shape. */
 int vgrid_set_launch(vgrid_t *g, const vgrid_launch *launch);
 int vgrid_get_launch(const vgrid_t *g, vgrid_launch *launch);
 

@@ -149,8 +149,11 @@ class VoronoiGrid:
 
     # -------------------------------------------------------------- launch
     def set_launch(self, lanes_per_ray=1, block=128, blocks_per_sm=0, fp64_lanes_per_ray=1, order=0):
-        """Launch shape of the traversal kernels; order: 1 = longest estimated
-        path first, -1 = the caller's order, 0 = automatic (see vgrid.h)."""
+        """Launch shape of the traversal kernels; without arguments the default,
+        in which calls with few rays use several lanes per ray. A form whose
+        lanes are 1 keeps that choice unless ``blocks_per_sm`` is set. order: 1 =
+        longest estimated path first, -1 = the caller's order, 0 = automatic (see
+        vgrid.h)."""
         l = _lib.Launch(int(lanes_per_ray), int(block), int(blocks_per_sm), int(fp64_lanes_per_ray), int(order))
         check(load().vgrid_set_launch(self._h, ctypes.byref(l)))
 

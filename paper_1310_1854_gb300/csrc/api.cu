@@ -91,7 +91,6 @@ struct vgrid {
     int64_t M = 0;
     vgrid_opts opts{};
     vgrid_launch launch{1, 128, 0, 1, 0};
-    bool launch_auto = true;         // no shape was set: lanes per ray follow the number of rays
     GridDev hd{};
     GridDev *d_desc = nullptr;
     float4 *d_site = nullptr;
@@ -603,7 +602,6 @@ int vgrid_set_launch(vgrid_t *g, const vgrid_launch *l) {
     if (!g) return fail(VGRID_ERR_ARG, "null grid");
     if (!l) {
         g->launch = vgrid_launch{1, 128, 0, 1, 0};
-        g->launch_auto = true;
         return VGRID_OK;
     }
     if (!valid_lpr(l->lanes_per_ray)) return fail(VGRID_ERR_ARG, "lanes_per_ray must be 1, 2, 4 or 8");
@@ -613,7 +611,6 @@ int vgrid_set_launch(vgrid_t *g, const vgrid_launch *l) {
     if (l->blocks_per_sm < 0) return fail(VGRID_ERR_ARG, "blocks_per_sm must be >= 0");
     if (l->order < -1 || l->order > 1) return fail(VGRID_ERR_ARG, "order must be -1, 0 or 1");
     g->launch = *l;
-    g->launch_auto = false;
     return VGRID_OK;
 }
 
@@ -778,8 +775,8 @@ int precision_row(int precision) {
     return precision == VGRID_FP64 ? 1 : precision == VGRID_FP32_EXACT ? 2 : 0;
 }
 
-// The launch shape of a call of N rays (lanes_per_ray resolved for the row).
-// Without a shape set by the caller the lanes per ray follow N: a launch whose
+// The launch shape of a call of N rays (lanes_per_ray resolved for the row). With
+// lanes_per_ray 1 and blocks_per_sm 0 the lanes per ray follow N: a launch whose
 // rays do not fill the lanes lasts as long as its longest ray, a chain of
 // dependent loads per crossing that several lanes shorten. R is the rays one
 // lane each keeps resident (136,192 for float32 tau). Per call, us, with
@@ -800,17 +797,17 @@ int precision_row(int precision) {
 // 1630 / 1324), and single-warp blocks while they do not fill the SMs (the
 // float64 pipes of all SMs then share the rays evenly: 60,000 rays 1.28 -> 1.17
 // ms).
+// Whether the lanes are the call's to choose is read off the shape itself, not
+// kept beside it, so that a shape read and set again is the same shape, and one
+// form's lanes can be set without fixing the other's.
 vgrid_launch shape_for(const vgrid_t *g, int row, int mode, int64_t N, bool enter = false) {
     vgrid_launch L = g->launch;
-    if (!g->launch_auto) {
-        if (row == 1 && L.fp64_lanes_per_ray) L.lanes_per_ray = L.fp64_lanes_per_ray;
-        return L;
-    }
-    L.lanes_per_ray = 1;
+    if (row == 1 && L.fp64_lanes_per_ray) L.lanes_per_ray = L.fp64_lanes_per_ray;
+    if (L.lanes_per_ray != 1 || L.blocks_per_sm != 0) return L;
     const double R = (double)persistent_blocks(kernels(1).get(row, mode), L, g->sms, INT64_MAX / 16) * L.block;
     if (row == 1) {
         L.lanes_per_ray = N <= 0.04 * R ? 8 : N <= 0.15 * R || (N > R && N <= 1.25 * R) ? 2 : 1;
-        if (N * L.lanes_per_ray < R) L.block = 32;
+        if (L.block == 128 && N * L.lanes_per_ray < R) L.block = 32;
     } else {
         const double f8 = enter ? 0.11 : 0.22, f4 = enter ? 0.27 : 0.75, f2 = enter ? 0.45 : 1.4;
         L.lanes_per_ray = N <= f8 * R ? 8 : N <= f4 * R ? 4 : N <= f2 * R ? 2 : 1;

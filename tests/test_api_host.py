@@ -133,3 +133,85 @@ int main() {
 """)
     nomem, cuda, ok = out[3].split()
     assert out[:3] == [f"{nomem} 0 0", f"{cuda} 0 0", f"{ok} 0 0"]
+
+
+SHAPES = r"""
+// kernels are numbers: lanes, then row, then mode
+namespace vg {
+static void table(KernelSet &k, int lanes) {
+    for (int r = 0; r < 3; r++)
+        for (int m = 0; m < NUM_MODES; m++) k.fn[r][m] = (const void *)(uintptr_t)(1000 * lanes + 100 * r + m);
+}
+void kernel_table_lpr1(KernelSet &k) { table(k, 1); }
+void kernel_table_lpr2(KernelSet &k) { table(k, 2); }
+void kernel_table_lpr4(KernelSet &k) { table(k, 4); }
+void kernel_table_lpr8(KernelSet &k) { table(k, 8); }
+void count_launches(int64_t) {}
+cudaError_t launch_locate(const LocateArgs &, int, int, cudaStream_t) { return cudaSuccess; }
+}  // namespace vg
+static int lanes, block;
+extern "C" {
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, int b, size_t) {
+    *n = 1024 / b;
+    return cudaSuccess;
+}
+cudaError_t cudaLaunchKernel(const void *f, dim3, dim3 b, void **, size_t, cudaStream_t) {
+    lanes = (int)((uintptr_t)f / 1000);
+    block = b.x;
+    return cudaSuccess;
+}
+}
+static vgrid_t *g;
+static void show(const char *what) {
+    static double o[3], d[3], tau[1];
+    printf("%s", what);
+    for (int p : {VGRID_FP32_RECHECK, VGRID_FP32_EXACT, VGRID_FP64}) {
+        vgrid_trace(g, o, d, 64, p, VGRID_TAU, tau, nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr);
+        printf(" %d/%d", lanes, block);
+    }
+    printf("\n");
+}
+static void set(int l, int b, int n, int l64, int order) {
+    const vgrid_launch s = {l, b, n, l64, order};
+    vgrid_set_launch(g, &s);
+}
+int main() {
+    const double S[] = {0.125, 0.25, 0.375, -0.5, 0.25, 0.0}, box[] = {-1, -1, -1, 1, 1, 1};
+    vgrid_opts o;
+    vgrid_default_opts(&o);
+    vgrid_create(S, 2, box, &o, &g);
+    vgrid_launch was, now;
+    show("new");
+    vgrid_get_launch(g, &was);
+    vgrid_set_launch(g, &was);
+    show("set what get returned");
+    set(4, 256, 2, 2, 0);
+    show("4 and 2 lanes");
+    set(was.lanes_per_ray, was.block, was.blocks_per_sm, was.fp64_lanes_per_ray, was.order);
+    show("restored");
+    set(was.lanes_per_ray, 256, 0, 4, was.order);
+    show("float64 tuned");
+    set(2, 256, 0, was.fp64_lanes_per_ray, was.order);
+    show("float32 tuned");
+    vgrid_set_launch(g, nullptr);
+    show("reset");
+    set(1, 128, 0, 1, -1);
+    show("caller's order");
+    set(1, 128, 8, 1, 0);
+    show("one lane");
+    vgrid_get_launch(g, &now);
+    printf("%d %d\n", was.lanes_per_ray, now.blocks_per_sm);
+    return 0;
+}
+"""
+
+
+def test_launch_shape_read_and_set_again(tmp_path):
+    """A call of few rays (64 of the 4096 resident ones) gets several lanes per
+    ray: on a new grid, after its shape is read and set again or restored, and
+    for the form whose lanes were left alone."""
+    out = _run(tmp_path, SHAPES)
+    auto = "8/128 8/128 8/32"
+    assert out[:10] == ["new " + auto, "set what get returned " + auto, "4 and 2 lanes 4/256 4/256 2/256",
+                        "restored " + auto, "float64 tuned 8/256 8/256 4/256", "float32 tuned 2/256 2/256 8/256",
+                        "reset " + auto, "caller's order " + auto, "one lane 1/128 1/128 1/128", "1 8"]
