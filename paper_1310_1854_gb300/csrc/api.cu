@@ -511,7 +511,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     hd.max_steps = o.max_steps;
     hd.zmax = o.zero_run_max;
     hd.domain = o.domain;
-    hd.pad1 = 0;
+    hd.lslack = hd.scale < 0x1p63 ? 0x1p-70f : std::numeric_limits<float>::infinity();
     for (int c = 0; c < 4; c++) hd.sph[c] = o.domain == VGRID_DOMAIN_SPHERE ? o.sphere[c] : 0.0;
     if (e == cudaSuccess) e = cudaMemcpy(g->d_desc, &hd, sizeof(GridDev), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {

@@ -103,7 +103,9 @@ struct GridDev {
     double scale;             // max |coordinate| of the box + diagonal
     int64_t max_steps;
     int32_t domain;           // VGRID_DOMAIN_BOX or VGRID_DOMAIN_SPHERE
-    int32_t pad1;
+    float lslack;             // C(r): off the bound that stops the scan of a block list. 2^-70 covers square
+                              // roots of sums rounded in the subnormal range; infinite (no stop) where a
+                              // sum of squares may overflow, whose root would bound nothing
     double sph[4];            // spherical domain: centre and radius
 };
 

@@ -461,8 +461,8 @@ __device__ __forceinline__ int locate_point(const GridDev *gp, const LocPt P, bo
             rp = __fsqrt_rn(__fmaf_rn(ez, ez, __fmaf_rn(ey, ey, __fmul_rn(ex, ex))));
         }
         // |p - c| rounded up, plus p's low words: subtracted from the bound
-        // (2^-70: square roots of sums rounded in the subnormal range)
-        const float slack = __fadd_ru(__fmul_ru(rp, 1.0f + 16.0f * kU), __fmaf_ru(4.0f * kU, X, 0x1p-70f));
+        // (lslack: see GridDev)
+        const float slack = __fadd_ru(__fmul_ru(rp, 1.0f + 16.0f * kU), __fmaf_ru(4.0f * kU, X, gp->lslack));
         for (int i = beg; i < end; i += 2) {
             float4 q[2];
             if (PAIRS) {
@@ -492,7 +492,8 @@ __device__ __forceinline__ int locate_point(const GridDev *gp, const LocPt P, bo
                 }
             }
         }
-        if (i1 >= 0 && D2 == __int_as_float(0x7f800000)) return i1;  // a single candidate
+        // a single candidate, or sums that overflowed: those are above 2^127
+        if (i1 >= 0 && D2 == __int_as_float(0x7f800000) && D1 < 0x1p126f) return i1;
         const float s1 = sqrtf(D1), s2 = sqrtf(D2);
         const float E1 = __fmaf_rn(1.0001f * kU, __fmaf_rn(10.0f, D1, 4.0f * X * s1), 0x1p-140f);
         const float E2 = __fmaf_rn(1.0001f * kU, __fmaf_rn(10.0f, D2, 4.0f * X * s2), 0x1p-140f);
