@@ -401,6 +401,14 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     g->device = dev;
     cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = cudaSuccess;
+    GridDev &hd = g->hd;
+    const double dx = bbox[3] - bbox[0], dy = bbox[4] - bbox[1], dz = bbox[5] - bbox[2];
+    const double diag = std::sqrt(dx * dx + dy * dy + dz * dz);
+    double dmax = 0;
+    for (int c = 0; c < 6; c++) dmax = std::max(dmax, std::fabs(bbox[c]));
+    hd.scale = dmax + diag;
+    hd.ushift = vg::unit_shift(hd.scale);
+    hd.unit = std::ldexp(1.0f, hd.ushift);
     // The device arrays (cell blocks of both forms, block lists, coarse density
     // grid), written by the device from the cells. Absolute cell blocks (offsets
     // A): header (caller id, count, rho = 1, F), then one record per neighbour
@@ -428,7 +436,7 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
                 site4[i] = make_float4((float)Si[3 * i], (float)Si[3 * i + 1], (float)Si[3 * i + 2], 0.0f);
         });
         vg::block_dims(bbox, M, o.blocks_per_site, g->blocks.dim);
-        vg::LayoutIn in{M, g->sms, bbox, {}, {}, site4.data(), g->perm.data(), g->cells.off.data(), g->cells.idx.data(),
+        vg::LayoutIn in{M, g->sms, bbox, hd.unit, {}, {}, site4.data(), g->perm.data(), g->cells.off.data(), g->cells.idx.data(),
                         g->cells.bbox.data(), left.off, left.idx, left.bbox};
         for (int c = 0; c < 3; c++) {
             in.bdim[c] = g->blocks.dim[c];
@@ -469,7 +477,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
     VG_ALLOC(g->d_stats, 1);
 #undef VG_ALLOC
 
-    GridDev &hd = g->hd;
     hd.site = g->d_site;
     hd.cells = g->d_cells;
     hd.rel = g->d_rel;
@@ -485,7 +492,6 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, g->device);
         hd.ospatial = (double)g->rel_bytes > 0.5 * (double)l2 ? 16 : 1;
     }
-    double dmax = 0;
     for (int c = 0; c < 3; c++) {
         hd.lo[c] = bbox[c];
         hd.hi[c] = bbox[3 + c];
@@ -499,15 +505,11 @@ int vgrid_create(const double *sites, int64_t M, const double bbox[6], const vgr
         hd.fbw[c] = (float)((bbox[3 + c] - bbox[c]) / g->blocks.dim[c]);
         hd.ddim[c] = ddim[c];
         hd.dscale[c] = (float)((double)ddim[c] / (bbox[3 + c] - bbox[c]));
-        dmax = std::max(dmax, std::max(std::fabs(bbox[c]), std::fabs(bbox[3 + c])));
     }
-    const double dx = bbox[3] - bbox[0], dy = bbox[4] - bbox[1], dz = bbox[5] - bbox[2];
-    const double diag = std::sqrt(dx * dx + dy * dy + dz * dz);
     hd.M = (int32_t)M;
     hd.kappa = 1.0f;
     hd.eps64 = 1e-12 * diag;
     hd.eps32 = 1e-6 * diag;
-    hd.scale = dmax + diag;
     hd.max_steps = o.max_steps;
     hd.zmax = o.zero_run_max;
     hd.domain = o.domain;

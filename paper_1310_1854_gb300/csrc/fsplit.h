@@ -61,15 +61,15 @@ VG_HD bool split_double_int(double x, float &hi, float &lo) {
     return true;
 }
 
-// x as float32, cut to its top 24 significant bits (error below 2^-23 |x|) with
-// integer operations; |x| < 2^-126 gives 0, and values beyond float32's range
-// (inf and NaN among them) are converted in float64.
-VG_HD float dtrunc(double x) {
+// x 2^by as float32, cut to its top 24 significant bits (error below 2^-23 of it)
+// with integer operations; below 2^-126 it is 0. Beyond float32's range (inf and
+// NaN among them) x is converted in float64, or with `by` is infinite.
+VG_HD float dtrunc(double x, int by = 0) {
     const uint64_t t = dbits(x);
     const uint32_t h = (uint32_t)(t >> 32);
-    const uint32_t e = (h >> 20) & 0x7ffu;
-    if (e - 897u > 253u) return e <= 896u ? 0.0f : (float)x;
-    return fbits((h & 0x80000000u) | (((h & 0x7fffffffu) - (896u << 20)) << 3) | ((uint32_t)t >> 29));
+    const int e = (int)((h >> 20) & 0x7ffu) + by;
+    if ((uint32_t)e - 897u > 253u) return e <= 896 ? 0.0f : by == 0 ? (float)x : fbits((h & 0x80000000u) | 0x7f800000u);
+    return fbits((h & 0x80000000u) | (((h & 0x7fffffffu) + (uint32_t)(by - 896) * (1u << 20)) << 3) | ((uint32_t)t >> 29));
 }
 
 // (double)x with integer operations where x is normal

@@ -4,6 +4,8 @@
 
 #include <vector_types.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <functional>
@@ -50,6 +52,12 @@ void parallel_for(int64_t n, int threads, int64_t grain, const std::function<voi
 void block_dims(const double *box, int64_t M, double blocks_per_site, int32_t *dim);
 void build_blocks(const double *box, const std::vector<double> &bbox, int64_t M, double blocks_per_site,
                   BlocksOut &out, int threads = 0);
+// GridDev::ushift of a box whose `scale` is given: 0 where the products of two
+// lengths in it are ordinary float32 numbers, else unit is about 1 / scale
+inline int unit_shift(double scale) {
+    const int e = std::ilogb(scale);
+    return e >= -20 && e <= 40 ? 0 : -std::min(std::max(e, -120), 120);
+}
 
 }  // namespace vg
 
@@ -106,6 +114,8 @@ struct GridDev {
     float lslack;             // C(r): off the bound that stops the scan of a block list. 2^-70 covers square
                               // roots of sums rounded in the subnormal range; infinite (no stop) where a
                               // sum of squares may overflow, whose root would bound nothing
+    float unit;               // power of two that the float64 form's float32 search takes lengths by
+    int32_t ushift;           // unit = 2^ushift
     double sph[4];            // spherical domain: centre and radius
 };
 

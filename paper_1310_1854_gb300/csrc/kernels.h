@@ -148,6 +148,7 @@ struct LayoutIn {
     int64_t M;
     int sms;
     const double *box;
+    float unit;                 // GridDev::unit
     int32_t bdim[3], ddim[3];   // block grid, coarse density grid
     const float4 *site4;        // (x, y, z, -) per cell
     const int32_t *perm;

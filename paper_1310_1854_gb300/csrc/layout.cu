@@ -37,6 +37,14 @@ __device__ __forceinline__ unsigned long long near_key(float d2, int id) {
     return ((unsigned long long)__float_as_uint(d2) << 32) | (unsigned)id;
 }
 
+// |unit n|^2 with the operations of the search's early stop
+__device__ __forceinline__ float norm2(float unit, float x, float y, float z) {
+    x = __fmul_rn(unit, x);
+    y = __fmul_rn(unit, y);
+    z = __fmul_rn(unit, z);
+    return __fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x)));
+}
+
 // entries of a cell's two blocks: 1 + neighbours and walls; 2 + cell
 // neighbours, at least four and an even count
 __global__ void cell_sizes_kernel(const int64_t *off, const int32_t *idx, int64_t M, int64_t *a, int64_t *f) {
@@ -63,7 +71,7 @@ __global__ void sites_kernel(const float4 *site, const int64_t *foffs, int64_t M
 __global__ void __launch_bounds__(32 * kWarps) cell_blocks_kernel(const float4 *site, const int32_t *perm,
                                                                   const int64_t *off, const int32_t *idx, int64_t M,
                                                                   const int64_t *aoffs, const int64_t *foffs,
-                                                                  float4 *cells, float4 *rel, int *big) {
+                                                                  float unit, float4 *cells, float4 *rel, int *big) {
     const int lane = threadIdx.x & 31;
     for (int64_t i = warp_index(); i < M; i += warp_count()) {
         const int64_t b = off[i];
@@ -92,15 +100,14 @@ __global__ void __launch_bounds__(32 * kWarps) cell_blocks_kernel(const float4 *
             if (q < n) cells[A + 1 + q] = r;
             int rank = ncell + __popc(cm & ((1u << lane) - 1u));
             if (sort) {
-                const unsigned long long key =
-                    near_key(__fmaf_rn(d.z, d.z, __fmaf_rn(d.y, d.y, __fmul_rn(d.x, d.x))), j);
+                const unsigned long long key = near_key(norm2(unit, d.x, d.y, d.z), j);
                 rank = 0;
                 for (int t = 0; t < n; t++) {
                     const int k = idx[b + t];
                     if (k < 0) continue;
                     const float4 s = site[k];
                     const float x = __fsub_rn(s.x, p.x), y = __fsub_rn(s.y, p.y), z = __fsub_rn(s.z, p.z);
-                    rank += near_key(__fmaf_rn(z, z, __fmaf_rn(y, y, __fmul_rn(x, x))), k) < key;
+                    rank += near_key(norm2(unit, x, y, z), k) < key;
                 }
             }
             if (cell) rel[F + 2 + rank] = d;
@@ -425,8 +432,8 @@ int build_layout(const LayoutIn &in, LayoutOut &out, std::string &err) {
     out.ncells = na + 8;
     out.nrel = nf + 8;
     sites_kernel<<<blocks_for(M, 256, in.sms), 256>>>(s4, foffs, M, out.site);
-    cell_blocks_kernel<<<blocks_for(M, kWarps, in.sms), wb>>>(s4, out.perm, off, idx, M, aoffs, foffs, out.cells, out.rel,
-                                                             reinterpret_cast<int *>(nbig + 1));
+    cell_blocks_kernel<<<blocks_for(M, kWarps, in.sms), wb>>>(s4, out.perm, off, idx, M, aoffs, foffs, in.unit, out.cells,
+                                                             out.rel, reinterpret_cast<int *>(nbig + 1));
     tail_kernel<<<1, 8>>>(out.cells, na, out.rel, nf);
     // coarse density grid
     BlockDev dg = g;

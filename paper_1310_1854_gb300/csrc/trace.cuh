@@ -530,17 +530,23 @@ struct Cand32 {
 //   |num~ - n.w|  <= dnum = N (4u N + 8u |r~|_1 + 2 e_r),   w = n/2 - r
 // dden and dnum are the same for every plane of the cell (computed once per
 // crossing from N).
+// In units where n.n leaves float32's range the float64 form searches with
+// lengths times a power of two, `unit` (GridDev): r, w, num, s and the bounds on
+// them are scaled (half = unit / 2), n, k and den are not. The float32 forms have
+// half = 1/2. 3 10^5 rays on the 10^5-site disk in units of 2^66 (a kiloparsec in
+// metres) take 1.8 ms instead of 19.4 with a float64 search per crossing, as many
+// as in units of 1 but for the start cells; so from 2^-80 up to 2^110.
 struct Plane32 {
     float num, den, dnum, dden;
 };
 
-__device__ __forceinline__ Plane32 plane32(float4 q, float rx, float ry, float rz, float dnum, float dden, float Kx,
-                                           float Ky, float Kz) {
+__device__ __forceinline__ Plane32 plane32(float4 q, float half, float rx, float ry, float rz, float dnum, float dden,
+                                           float Kx, float Ky, float Kz) {
     Plane32 p;
     const float nx = q.x, ny = q.y, nz = q.z;
     p.den = __fmaf_rn(nz, Kz, __fmaf_rn(ny, Ky, __fmul_rn(nx, Kx)));
     p.dden = dden;
-    const float wx = __fmaf_rn(0.5f, nx, -rx), wy = __fmaf_rn(0.5f, ny, -ry), wz = __fmaf_rn(0.5f, nz, -rz);
+    const float wx = __fmaf_rn(half, nx, -rx), wy = __fmaf_rn(half, ny, -ry), wz = __fmaf_rn(half, nz, -rz);
     p.num = __fmaf_rn(nz, wz, __fmaf_rn(ny, wy, __fmul_rn(nx, wx)));
     p.dnum = dnum;
     return p;
@@ -574,9 +580,9 @@ __device__ __forceinline__ float rcp_ftz(float b) {
 // costs nothing more. Positions past the count (several lanes per ray) are
 // masked by `valid`.
 template <bool KEEP>
-__device__ __forceinline__ void consider32(int pos, bool valid, float4 q, float rx, float ry, float rz, float dnumK,
-                                           float dden, float Kx, float Ky, float Kz, Cand32 &c) {
-    const Plane32 p = plane32(q, rx, ry, rz, dnumK, dden, Kx, Ky, Kz);
+__device__ __forceinline__ void consider32(int pos, bool valid, float4 q, float half, float rx, float ry, float rz,
+                                           float dnumK, float dden, float Kx, float Ky, float Kz, Cand32 &c) {
+    const Plane32 p = plane32(q, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz);
     const float num_lo = fmaxf(__fmaf_rd(p.num, kDivLo, -dnumK), 0.0f);
     const float den_hi = __fadd_ru(p.den, p.dden);
     float lower;
@@ -632,7 +638,14 @@ struct Stop32 {
     float step;          // S above the smallest lower bound
 };
 
-__device__ __forceinline__ bool beyond(float4 q, float S, const Stop32 &e) {
+// UNIT: lengths but n come scaled (see Plane32)
+template <bool UNIT>
+__device__ __forceinline__ bool beyond(float4 q, float unit, float S, const Stop32 &e) {
+    if (UNIT) {
+        q.x = __fmul_rn(unit, q.x);
+        q.y = __fmul_rn(unit, q.y);
+        q.z = __fmul_rn(unit, q.z);
+    }
     const float nn = __fmaf_rn(q.z, q.z, __fmaf_rn(q.y, q.y, __fmul_rn(q.x, q.x)));
     const float v = __fmaf_rn(S, __fadd_rn(S, e.rk2), e.rr);
     return __fmul_rn(fmaxf(v, e.rrm), kStopHold) < nn;
@@ -645,11 +658,12 @@ constexpr int kWallWin = -1;  // Cand32::w1 when the wall ahead is the smallest 
 // per ray the caller loads the first four (f0..f3) together with the header,
 // so they do not wait for the count, no position is ever past the count, and
 // the wall ahead (lower bound lw) is the first candidate.
-template <int LPR>
+template <int LPR, bool UNIT>
 __device__ __forceinline__ void exit32(const float4 *recs, int cnt, float4 f0, float4 f1, float4 f2, float4 f3,
-                                       float rx, float ry, float rz, float dnumK, float dden, float Kx, float Ky,
+                                       float unit, float rx, float ry, float rz, float dnumK, float dden, float Kx, float Ky,
                                        float Kz, float lw, const Stop32 &e, unsigned gmask, int gl, int gbase,
                                        Cand32 &c) {
+    const float half = UNIT ? 0.5f * unit : 0.5f;
     c.L1 = LPR == 1 ? lw : __int_as_float(0x7f800000);
     c.L2 = __int_as_float(0x7f800000);
     c.p1 = 0;
@@ -657,15 +671,15 @@ __device__ __forceinline__ void exit32(const float4 *recs, int cnt, float4 f0, f
     c.den1 = 1.f;
     c.w1 = kWallWin;
     if (LPR == 1) {
-        consider32<true>(1, true, f0, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-        consider32<true>(2, true, f1, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-        consider32<true>(3, true, f2, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-        consider32<true>(4, true, f3, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+        consider32<true>(1, true, f0, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+        consider32<true>(2, true, f1, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+        consider32<true>(3, true, f2, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+        consider32<true>(4, true, f3, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
         const float nan = __int_as_float(0x7fc00000);
         float4 last = f3;
         for (int p = 5; p <= cnt; p += 4) {
             const float S = __fadd_rn(c.L1, e.step);
-            if (beyond(last, S, e)) {
+            if (beyond<UNIT>(last, unit, S, e)) {
                 c.L2 = fminf(c.L2, S);
                 break;
             }
@@ -673,10 +687,10 @@ __device__ __forceinline__ void exit32(const float4 *recs, int cnt, float4 f0, f
             float4 q0, q1, q2 = make_float4(nan, nan, nan, nan), q3 = q2;
             ldg_pair(recs + p, q0, q1);
             if (p + 2 <= cnt) ldg_pair(recs + p + 2, q2, q3);
-            consider32<true>(p, true, q0, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<true>(p + 1, true, q1, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<true>(p + 2, true, q2, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<true>(p + 3, true, q3, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<true>(p, true, q0, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<true>(p + 1, true, q1, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<true>(p + 2, true, q2, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<true>(p + 3, true, q3, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
             last = q3;
         }
     } else {
@@ -688,10 +702,10 @@ __device__ __forceinline__ void exit32(const float4 *recs, int cnt, float4 f0, f
             const float4 q1 = p1 <= cnt ? __ldg(recs + p1) : pad;
             const float4 q2 = p2 <= cnt ? __ldg(recs + p2) : pad;
             const float4 q3 = p3 <= cnt ? __ldg(recs + p3) : pad;
-            consider32<false>(p0, true, q0, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<false>(p1, p1 <= cnt, q1, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<false>(p2, p2 <= cnt, q2, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
-            consider32<false>(p3, p3 <= cnt, q3, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<false>(p0, true, q0, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<false>(p1, p1 <= cnt, q1, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<false>(p2, p2 <= cnt, q2, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
+            consider32<false>(p3, p3 <= cnt, q3, half, rx, ry, rz, dnumK, dden, Kx, Ky, Kz, c);
         }
     }
     if (LPR > 1) {
@@ -795,6 +809,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
     Hot h{a.g1.cells, a.g1.rel, a.g1.site};
     float kappa = a.g1.kappa;
     int max_steps = (int)min(a.g1.max_steps, (int64_t)0x7fffffff);
+    const float unit = FP64 ? a.g1.unit : 1.0f;
     // float64 form: current point and direction, the distance gone in float32
     // and the bounds on the boundary's distance (both only bound the wall)
     double r64[3] = {0, 0, 0}, k64[3] = {0, 0, 0};
@@ -1086,9 +1101,9 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             // the current point in the frame of the site, to within 2u|r| + e_r
             float rx, ry, rz;
             if (FP64) {
-                rx = dtrunc(__dsub_rn(r64[0], fexact(pmx)));
-                ry = dtrunc(__dsub_rn(r64[1], fexact(pmy)));
-                rz = dtrunc(__dsub_rn(r64[2], fexact(pmz)));
+                rx = dtrunc(__dsub_rn(r64[0], fexact(pmx)), a.g1.ushift);
+                ry = dtrunc(__dsub_rn(r64[1], fexact(pmy)), a.g1.ushift);
+                rz = dtrunc(__dsub_rn(r64[2], fexact(pmz)), a.g1.ushift);
             } else {
                 rx = local_coord(R0h_(0), R0l_(0), Kh[0], Kl_(0), th, tl, pmx);
                 ry = local_coord(R0h_(1), R0l_(1), Kh[1], Kl_(1), th, tl, pmy);
@@ -1097,16 +1112,17 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             const float r1 = __fadd_rn(__fadd_rn(fabsf(rx), fabsf(ry)), fabsf(rz));
             // the error terms of r and of the wall distance from t_max (no
             // shared-memory reads)
-            const float tmax_h = FP64 ? wlo : tmh_;
+            const float tmax_h = FP64 ? fmaxf(wlo, 0.0f) : tmh_;
             const float scale = BATCH ? (float)gp->scale : (float)a.g1.scale;
             // the float64 form's own rounding, 2^-29 of these terms, goes into
             // them, and dtrunc's cut at 2^-126 into e_r
-            const float er = __fmaf_rn(16.0f * kU2, __fadd_rn(scale, tmax_h), FP64 ? 0x1p-124f : 0.0f);
+            const float er = __fmaf_rn(FP64 ? 16.0f * kU2 * unit : 16.0f * kU2, __fadd_rn(scale, tmax_h), FP64 ? 0x1p-124f : 0.0f);
             const float rr = __fmaf_rn(FP64 ? 1.0001f * kCB : kCB, r1, 2.0f * er);
             const float n1m = hdr1.z;  // the cell's bound on |n|_1
+            const float n1u = FP64 ? __fmul_rn(unit, n1m) : n1m;
             // the rounding bound of den~ plus 2^-126 (see consider32)
             const float dden = __fadd_ru(__fmul_ru(FP64 ? 1.0001f * kCDen : kCDen, n1m), kDivMin);
-            const float dnum = __fmul_ru(n1m, __fmaf_ru(FP64 ? 1.0001f * kCA : kCA, n1m, rr));
+            const float dnum = __fmul_ru(n1m, __fmaf_ru(FP64 ? 1.0001f * kCA : kCA, n1u, rr));
             // the wall ahead is one more candidate: s_w = t_max - t
             float sw, lw, uw;
             if (FP64) {
@@ -1114,8 +1130,8 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 // 24 bits and added with one rounding)
                 const float Eg = __fmul_ru((float)(steps + 8) * (2.0f * kU), gone);
                 sw = 0.f;
-                lw = __fsub_rd(__fsub_rd(wlo, gone), Eg);
-                uw = steps < 32768 ? __fadd_ru(__fsub_ru(whi, gone), Eg) : __int_as_float(0x7f800000);
+                lw = __fmul_rd(unit, __fsub_rd(__fsub_rd(wlo, gone), Eg));
+                uw = steps < 32768 ? __fmul_ru(unit, __fadd_ru(__fsub_ru(whi, gone), Eg)) : __int_as_float(0x7f800000);
                 if (steps >= 32768) lw = 0.f;  // the bounds hold no longer: search in float64
             } else {
                 float swl;
@@ -1130,10 +1146,10 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             e.rk2 = 2.0f * __fmaf_rn(rz, Kh[2], __fmaf_rn(ry, Kh[1], __fmul_rn(rx, Kh[0])));
             const float er18 = 0x1p18f * er;
             e.rrm = fmaxf(e.rr, __fmul_rn(er18, er18));
-            e.step = __fmul_rn(n1m, kStopStep);
+            e.step = __fmul_rn(n1u, kStopStep);
             Cand32 c;
-            exit32<LPR>(recs, cnt, f0, f1, f2, f3, rx, ry, rz, __fmul_ru(dnum, kDivLo), dden, Kh[0], Kh[1], Kh[2], lw,
-                        e, gmask, gl, gbase, c);
+            exit32<LPR, FP64>(recs, cnt, f0, f1, f2, f3, unit, rx, ry, rz, __fmul_ru(dnum, kDivLo), dden, Kh[0], Kh[1],
+                              Kh[2], lw, e, gmask, gl, gbase, c);
             bool wall_wins = LPR == 1 && c.w1 == kWallWin;
             if (LPR > 1) {
                 if (lw < c.L1) {
@@ -1156,7 +1172,7 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 } else {
                     // the winner's terms again (same operations, same values)
                     qw = __ldg(recs + c.p1);
-                    w1 = plane32(qw, rx, ry, rz, dnum, dden, Kh[0], Kh[1], Kh[2]);
+                    w1 = plane32(qw, 0.5f * unit, rx, ry, rz, dnum, dden, Kh[0], Kh[1], Kh[2]);
                 }
                 const float den_lo = __fsub_rd(w1.den, w1.dden);
                 const float num_hi = fmaxf(__fadd_ru(w1.num, w1.dnum), 0.0f);
@@ -1171,13 +1187,17 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
                 Cand32 f{lw, __int_as_float(0x7f800000), 0, 0.f, 1.f, kWallWin};
 #pragma unroll 1
                 for (int p = 1; p <= cnt; p++)
-                    consider32<true>(p, true, __ldg(recs + p), rx, ry, rz, __fmul_ru(dnum, kDivLo), dden, Kh[0], Kh[1],
-                                     Kh[2], f);
+                    consider32<true>(p, true, __ldg(recs + p), 0.5f * unit, rx, ry, rz, __fmul_ru(dnum, kDivLo), dden,
+                                     Kh[0], Kh[1], Kh[2], f);
                 apart = f.w1 == c.w1 && upper < f.L2;
             }
             // the float64 form takes any scale: where products of the cell's
-            // differences would leave float32's normal range it searches itself
-            if (FP64) apart = apart && n1m > 0x1p-50f && n1m < 0x1p60f;
+            // differences leave float32's normal range all the same (num~ is about
+            // n.n unit, the squares of the early stop n.n unit^2) it searches itself
+            if (FP64) {
+                const float nn = __fmul_rn(n1m, n1u);
+                apart = apart && n1u > 0x1p-50f && nn > 0x1p-100f && nn < 0x1p120f;
+            }
             if (apart && FP64) {
                 // the exit is known: Eq. 4 (or Eq. 5, or the sphere) in float64
                 // for it alone, with the operations of a search of the cell

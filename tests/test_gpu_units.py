@@ -49,3 +49,29 @@ def test_cells_of_points_in_every_unit(place):
                 c = vg.locate(dev(P * scale), precision=prec)
                 want = c if want is None else want
                 assert torch.equal(c, want), (p, per_site, prec)
+
+
+@pytest.mark.parametrize("place", ["uniform", "disk", "ball"])
+def test_float64_results_scale_with_the_unit(place):
+    from paper_1310_1854_gb300 import VoronoiGrid
+    g, rays, sphere = _grid(place)
+    D = dev(rays.dir)
+
+    def run(scale):
+        kw = {} if sphere is None else {"sphere": tuple(sphere * scale)}
+        vg = VoronoiGrid(g.sites * scale, g.box * scale, **kw)
+        vg.set_density(dev(g.rho))
+        O = dev(rays.origin * scale)
+        out = []
+        for shape in ({"blocks_per_sm": 64}, {}, {"fp64_lanes_per_ray": 4}):
+            vg.set_launch(**shape)
+            r = vg.trace(O, D, precision="fp64", segments=True, status=True)
+            t = vg.trace(O, D, precision="fp64")
+            out.append((r.seg_off, r.seg_cell, r.status, r.seg_len / scale, r.tau / scale, t.tau / scale))
+        return out
+
+    want = run(1.0)
+    for p in (-105, -95, -70, -30, -21, 39, 42, 62, 64, 65, 66, 76, 95, 110):
+        for a, b in zip(run(2.0 ** p), want):
+            for i, (x, y) in enumerate(zip(a, b)):
+                assert torch.equal(x, y), (p, i)
