@@ -249,7 +249,11 @@ class VoronoiGrid:
             self._seg_per_ray = total / N
         cells, lens = cells[:total], lens[:total]
         if seg_capacity is None and cap > 1.5 * total + 4096:
-            cells, lens = cells.clone(), lens.clone()  # the lists do not keep a generous first guess alive
+            # the lists do not keep a generous first guess alive
+            try:
+                cells, lens = cells.clone(), lens.clone()
+            except torch.cuda.OutOfMemoryError:
+                pass  # no room for a second copy: the lists as they are
         return TraceResult(tau, seg_off, cells, lens, st, cs.as_dict())
 
     def trace_host(self, origin, direction, precision="fp32", out_tau=None, status=False, stats=False, chunk=0,
