@@ -383,6 +383,10 @@ int vgrid_segments_grad(vgrid_t *g, const int64_t *seg_off, const int32_t *seg_c
 int vgrid_interact(vgrid_t *g, const double *origin, const double *dir, int64_t N, const float *tau_int,
                    const float *weight, int32_t *cell, float *s, float *absorbed, vgrid_stream_t stream);
 
+/* Give back the chunk buffers of segment mode (the next call that needs them
+ * allocates them again). No call may be in flight on the grid. */
+int vgrid_trim(vgrid_t *g);
+
 /* Launch shape used by this grid's traversal kernels. NULL resets to the
  * built-in default, which a new grid has (1, 128, 0, 1, 0). Setting the shape
  * that vgrid_get_launch returned changes nothing. Results do not depend on the

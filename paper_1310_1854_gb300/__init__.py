@@ -26,6 +26,10 @@ __all__ = ["VoronoiGrid", "Batch", "TraceResult", "optical_depth", "probe_l2", "
 # entries that trace(..., segments=True) sizes its buffers for on a guess; a call
 # that would need more counts first
 _SEG_GUESS_MAX = 1 << 30
+# bytes of lists and work buffers that a first guess takes without a look at the
+# free memory, and of which the buffers may stay with the grid at that size (to
+# free and allocate 0.7 GB of them again costs a call about 0.6 ms)
+_SEG_SMALL = 1 << 32
 
 _PREC = {"fp64": _lib.FP64, "fp32": _lib.FP32_RECHECK, "fp32_exact": _lib.FP32_EXACT}
 
@@ -205,6 +209,7 @@ class VoronoiGrid:
                                   _ptr(st), sref, _stream(stream)))
             return TraceResult(tau, status=st, stats=cs.as_dict() if cs is not None else None)
         seg_off = torch.empty(N + 1, dtype=torch.int64, device=self.device)
+        first = False  # a first guess that takes much memory
         if seg_capacity is not None:
             cap = int(seg_capacity)
         else:
@@ -214,7 +219,9 @@ class VoronoiGrid:
             # measured on uniform, clumpy and disk sites)
             per_ray = 1.25 * self._seg_per_ray if self._seg_per_ray is not None else 1.25 * self.M ** (1 / 3) + 8.0
             cap = int(N * per_ray) + 1024
-            if cap > _SEG_GUESS_MAX:
+            first = self._seg_per_ray is None and self._seg_bytes(cap, N, prec) > _SEG_SMALL
+            if cap > _SEG_GUESS_MAX or (first and self._seg_bytes(cap, N, prec) >
+                                        torch.cuda.mem_get_info(self.device)[0] // 4):
                 cap = 0
 
         def lists(n):
@@ -249,12 +256,22 @@ class VoronoiGrid:
             self._seg_per_ray = total / N
         cells, lens = cells[:total], lens[:total]
         if seg_capacity is None and cap > 1.5 * total + 4096:
-            # the lists do not keep a generous first guess alive
+            # a generous first guess is not kept alive, by the grid (its work
+            # buffers, where they are large) or by the lists
+            if first:
+                check(lib.vgrid_trim(self._h))
             try:
                 cells, lens = cells.clone(), lens.clone()
             except torch.cuda.OutOfMemoryError:
                 pass  # no room for a second copy: the lists as they are
         return TraceResult(tau, seg_off, cells, lens, st, cs.as_dict())
+
+    @staticmethod
+    def _seg_bytes(cap, N, prec):
+        """Bytes of segment lists for ``cap`` entries and of the library's work
+        buffers for them (chunks of 8 slots, one started per ray)."""
+        slot, slots = (16 if prec == _lib.FP64 else 8), cap + 8 * min(N, cap)
+        return cap * (4 + slot // 2) + slots * slot + 12 * (slots // 8)
 
     def trace_host(self, origin, direction, precision="fp32", out_tau=None, status=False, stats=False, chunk=0,
                    stream=None, wait=True) -> TraceResult:

@@ -101,6 +101,7 @@ SIGNATURES = [
                                       c_void_p]),
     ("vgrid_set_launch", c_int32, [c_void_p, ctypes.POINTER(Launch)]),
     ("vgrid_get_launch", c_int32, [c_void_p, ctypes.POINTER(Launch)]),
+    ("vgrid_trim", c_int32, [c_void_p]),
     ("vgrid_batch_create", c_int32, [ctypes.POINTER(Rayset), c_int32, ctypes.POINTER(Launch),
                                      ctypes.POINTER(c_void_p)]),
     ("vgrid_batch_run", c_int32, [c_void_p, c_int32, ctypes.POINTER(Stats), c_void_p]),

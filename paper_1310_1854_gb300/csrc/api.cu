@@ -707,6 +707,22 @@ int ensure_scan(vgrid_t *g, int64_t N) {
     return VGRID_OK;
 }
 
+void free_slots(vgrid_t *g) {
+    if (g->d_slots) cudaFree(g->d_slots);
+    g->device_bytes -= g->slot_bytes;
+    g->d_slots = nullptr;
+    g->slot_bytes = 0;
+}
+
+void free_chunk_meta(vgrid_t *g) {
+    if (g->d_chunk_meta) cudaFree(g->d_chunk_meta);
+    if (g->d_chunk_inv) cudaFree(g->d_chunk_inv);
+    g->device_bytes -= g->meta_cap * (int64_t)(sizeof(int2) + sizeof(int32_t));
+    g->d_chunk_meta = nullptr;
+    g->d_chunk_inv = nullptr;
+    g->meta_cap = 0;
+}
+
 // chunk pool of segment mode: `chunks` chunks of kSegChunk slots of
 // slot_bytes, their (ray, position) records and the inverse map, and the
 // chunk offsets of N rays
@@ -722,21 +738,13 @@ int ensure_chunks(vgrid_t *g, int64_t N, int64_t chunks, int slot_bytes) {
     }
     const int64_t bytes = chunks * vg::kSegChunk * slot_bytes;  // a multiple of 64
     if (bytes > g->slot_bytes) {
-        if (g->d_slots) cudaFree(g->d_slots);
-        g->device_bytes -= g->slot_bytes;
-        g->d_slots = nullptr;
-        g->slot_bytes = 0;
+        free_slots(g);
         int rc = dmalloc(&g->d_slots, (size_t)(bytes / 16), g->device_bytes);
         if (rc) return rc;
         g->slot_bytes = bytes;
     }
     if (chunks > g->meta_cap) {
-        if (g->d_chunk_meta) cudaFree(g->d_chunk_meta);
-        if (g->d_chunk_inv) cudaFree(g->d_chunk_inv);
-        g->device_bytes -= g->meta_cap * (int64_t)(sizeof(int2) + sizeof(int32_t));
-        g->d_chunk_meta = nullptr;
-        g->d_chunk_inv = nullptr;
-        g->meta_cap = 0;
+        free_chunk_meta(g);
         int rc = dmalloc(&g->d_chunk_meta, (size_t)chunks, g->device_bytes);
         if (!rc) rc = dmalloc(&g->d_chunk_inv, (size_t)chunks, g->device_bytes);
         if (rc) return rc;
@@ -1070,6 +1078,15 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     if ((int64_t)h.cursor > chunks)  // cannot happen when the total fits (see above)
         return fail(VGRID_ERR_CUDA, "segment chunk pool ran out");
     return src;
+}
+
+int vgrid_trim(vgrid_t *g) {
+    if (!g) return fail(VGRID_ERR_ARG, "null grid");
+    if (g->device < 0) return VGRID_OK;
+    DeviceGuard dg(g->device);
+    free_slots(g);
+    free_chunk_meta(g);
+    return VGRID_OK;
 }
 
 int vgrid_trace_host(vgrid_t *g, const double *origin, const double *dir, int64_t N, int precision, void *tau,
