@@ -737,6 +737,7 @@ int build_cells_gpu(const double *S, int64_t M, const double *box, int threads, 
     };
     auto bad = [&](cudaError_t e, const char *what) {
         err = std::string("GPU cell construction: ") + what + ": " + cudaGetErrorString(e);
+        cudaGetLastError();  // or the next launch's check would report it
         cleanup();
         return -1;
     };

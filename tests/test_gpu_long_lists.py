@@ -35,3 +35,16 @@ def test_nearest_site_from_long_lists(where, n, per_site):
         vg = VoronoiGrid(S, gen.CUBE_BOX, blocks_per_site=per_site, reorder=reorder)
         for p in ("fp32", "fp64"):
             assert np.array_equal(vg.locate(dev(P), precision=p).cpu().numpy(), want), (reorder, p)
+
+
+@pytest.mark.parametrize("gpu_build", [False, True])
+def test_lists_that_are_refused(gpu_build):
+    """2^30 blocks and two entries each exceed what offsets hold: the error, and
+    a device that takes the next grid."""
+    from paper_1310_1854_gb300 import VGridError, VoronoiGrid
+    g = gen.make_uniform_grid(1000, 3)
+    rays = gen.uniform_rays(1000, 4)
+    with pytest.raises(VGridError, match="2\\^31"):
+        VoronoiGrid(g.sites, g.box, gpu_build=gpu_build, blocks_per_site=1.1e6)
+    tau = [VoronoiGrid(g.sites, g.box, gpu_build=b).trace(dev(rays.origin), dev(rays.dir)).tau for b in (gpu_build, False)]
+    assert torch.equal(*tau)
