@@ -204,11 +204,12 @@ void vgrid_default_opts(vgrid_opts *opts);
  *   sites  host, M x 3 float64 (x, y, z per site), all inside the closed box.
  *   bbox   host, 6 float64: xmin, ymin, zmin, xmax, ymax, zmax.
  *   opts   host, nullable (defaults).
- * On the host: the cell of every site is cut from the box by the bisector
- * half-spaces of nearby sites (Sect. 2.1), giving neighbour lists with walls,
- * cell volumes and bounding boxes; the bounding boxes fill a regular block grid
- * of candidate lists for C(r) (Sect. 2.3). The lists, the sites (float32) and
- * a default density rho = 1, kappa = 1 are then copied to the current device.
+ * The cell of every site is cut from the box by the bisector half-spaces of
+ * nearby sites (Sect. 2.1), on the host or with gpu_build on the current
+ * device, giving neighbour lists with walls, cell volumes and bounding boxes.
+ * On the device the bounding boxes then fill a regular block grid of candidate
+ * lists for C(r) (Sect. 2.3), and the lists and sites (float32) become the
+ * traversal's cell blocks, with a default density rho = 1, kappa = 1.
  * Errors: VGRID_ERR_ARG, VGRID_ERR_OUTSIDE (site outside box),
  * VGRID_ERR_DUP_SITE, VGRID_ERR_BUILD, VGRID_ERR_NOMEM, VGRID_ERR_CUDA.
  */

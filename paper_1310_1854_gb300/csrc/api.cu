@@ -801,12 +801,16 @@ int precision_row(int precision) {
 // 307 / 343, 75,000 315 / 330 / 364 / 476. Parallel rays of a detector, started
 // on the domain's face, are like them but cannot be told from others here: eight
 // lanes stop at 0.22 R, where they lose little (30,600 of them through a ball,
-// forward and adjoint, 959 / 928 / 985 / 1233). The float64 form repeats its float64 work in every lane, so it takes
-// more than one only for very few rays (10^4 rays on 1000 sites: 128 / 111 / 133 /
-// 172) and where one lane each would leave a short second wave (10^5 on the disk:
-// 1630 / 1324), and single-warp blocks while they do not fill the SMs (the
-// float64 pipes of all SMs then share the rays evenly: 60,000 rays 1.28 -> 1.17
-// ms).
+// forward and adjoint, 959 / 928 / 985 / 1233). The float64 form (R = 97,280) repeats its float64 work in every
+// lane, so it takes more than one only for very few rays and where one lane each
+// would leave a short second wave, and single-warp blocks while they do not fill
+// the SMs (the float64 pipes of all SMs then share the rays evenly). One against
+// two lanes at 1.02 / 1.1 / 1.24 R: 10^5 disk sites 1596 - 1479, 1643 - 1510, 1649 -
+// 1565; 10^4 disk sites 758 - 701, 781 - 734, 791 - 742; 20,000 in a ball 695 - 618,
+// 708 - 657, 743 - 726; 2 10^5 clumpy ones 1080 - 1042, 1092 - 1066, 1127 - 1123; 10^5
+// uniform ones 878 - 861, 893 - 887, 923 - 930. At 0.95 and 1.5 R one lane is better
+// on four of these five; at 0.1 R two are on all (0.92 of the time), and at 0.03 R
+// eight (0.67 to 0.88). Small blocks at 0.5 R: 0.89 to 0.96.
 // Whether the lanes are the call's to choose is read off the shape itself, not
 // kept beside it, so that a shape read and set again is the same shape, and one
 // form's lanes can be set without fixing the other's.
@@ -1050,7 +1054,7 @@ int vgrid_trace(vgrid_t *g, const double *origin, const double *dir, int64_t N, 
     }
     if ((rc = ensure_scan(g, N))) return rc;
     if ((rc = ensure_chunks(g, N, chunks, fp64 ? 16 : 8))) return rc;
-    // the chunk cursor sits with the counters, which the set-up kernel cleared
+    // the chunk cursor sits with the counters, which the start-cell kernel cleared
     unsigned long long *const cursor = reinterpret_cast<unsigned long long *>(
         reinterpret_cast<char *>(g->d_stats) + offsetof(StatsDev, cursor));
     a.seg_off = seg_off;

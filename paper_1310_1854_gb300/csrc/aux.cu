@@ -1,6 +1,6 @@
-// Auxiliary kernels of libvgrid: start-cell location (C(r), Sect. 2.3),
-// per-call set-up, density reordering and the prefix sum that turns
-// per-ray segment counts into offsets.
+// Auxiliary kernels of libvgrid: start-cell location (C(r), Sect. 2.3), which
+// also clears a call's counters, density reordering and the prefix sum that
+// turns per-ray segment counts into offsets.
 #include <algorithm>
 #include <atomic>
 

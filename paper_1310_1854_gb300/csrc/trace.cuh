@@ -31,7 +31,7 @@
 //    a plain C implementation with contraction disabled, the current point
 //    updated as r <- r + s k. On the 10^5-site disk one crossing in about 10^4 is
 //    searched in float64. The float64 pipe bounds the form: testing every plane
-//    that may face ahead in float64 took 17.0 ms per 10^6 rays there, 3.46 ms
+//    that may face ahead in float64 took 17.0 ms per 10^6 rays there, 3.30 ms
 //    now (about 50 float64 instructions per crossing instead of some 300).
 //  * float32: the length is the float32 quotient (or, with exact lengths, a
 //    float-pair one); the ray parameter t is kept as an unevaluated float pair,
