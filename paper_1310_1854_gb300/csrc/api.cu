@@ -808,9 +808,10 @@ int precision_row(int precision) {
 // two lanes at 1.02 / 1.1 / 1.24 R: 10^5 disk sites 1596 - 1479, 1643 - 1510, 1649 -
 // 1565; 10^4 disk sites 758 - 701, 781 - 734, 791 - 742; 20,000 in a ball 695 - 618,
 // 708 - 657, 743 - 726; 2 10^5 clumpy ones 1080 - 1042, 1092 - 1066, 1127 - 1123; 10^5
-// uniform ones 878 - 861, 893 - 887, 923 - 930. At 0.95 and 1.5 R one lane is better
-// on four of these five; at 0.1 R two are on all (0.92 of the time), and at 0.03 R
-// eight (0.67 to 0.88). Small blocks at 0.5 R: 0.89 to 0.96.
+// uniform ones 878 - 861, 893 - 887, 923 - 930. At 0.95 R one lane is better on all
+// five, at 1.5 R on the last three by 2 to 8 % (two lanes by 6 % on the disks). At
+// 0.1 R two lanes take 0.85 to 0.95 of one lane's time, at 0.03 R eight 0.68 to
+// 0.86; small blocks at 0.5 R 0.89 to 0.95.
 // Whether the lanes are the call's to choose is read off the shape itself, not
 // kept beside it, so that a shape read and set again is the same shape, and one
 // form's lanes can be set without fixing the other's.
