@@ -1127,8 +1127,9 @@ __global__ void __launch_bounds__(256) __maxnreg__((trace_max_regs<FP64, MODE, B
             float sw, lw, uw;
             if (FP64) {
                 // t is off by less than (steps + 2) 2u t (each length cut to
-                // 24 bits and added with one rounding)
-                const float Eg = __fmul_ru((float)(steps + 8) * (2.0f * kU), gone);
+                // 24 bits and added with one rounding), and by 2^-126 for each
+                // length below that, which the cut takes as 0
+                const float Eg = __fmul_ru((float)(steps + 8), __fmaf_ru(2.0f * kU, gone, 0x1p-125f));
                 sw = 0.f;
                 lw = __fmul_rd(unit, __fsub_rd(__fsub_rd(wlo, gone), Eg));
                 uw = steps < 32768 ? __fmul_ru(unit, __fadd_ru(__fsub_ru(whi, gone), Eg)) : __int_as_float(0x7f800000);
