@@ -171,7 +171,8 @@ typedef struct {
 typedef struct {
     int32_t lanes_per_ray;      /* 2, 4 or 8: so many lanes cooperate on one ray. 1 (default):
                                    one, or more in calls with too few rays to fill the GPU
-                                   that way; with blocks_per_sm > 0 always one */
+                                   that way; with blocks_per_sm > 0, and in a batch,
+                                   always one */
     int32_t block;              /* threads per block (multiple of 32, 32..256; default 128) */
     int32_t blocks_per_sm;      /* persistent blocks per SM; 0 = as many as fit */
     int32_t fp64_lanes_per_ray; /* the same for the float64 form; 0 = lanes_per_ray (default 1).
